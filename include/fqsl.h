@@ -268,7 +268,9 @@ FQSL_API fqsl_status fqsl_twist(fqsl_field field, const double *seeds_dev, long 
  * waits for the events of the last call and returns their durations in
  * milliseconds: ms[0] line tracer (lattice or seed list; the FP32 seed
  * pre-pass runs just before it and is not included), ms[1] tracer of the
- * rotated-S0 extra lines (0 if not launched), ms[2] Q assembly. Errors:
+ * rotated-S0 extra lines (0 if not launched; a timed FP32 call gives them a
+ * launch of their own, an untimed one traces them with the lattice), ms[2] Q
+ * assembly. Errors:
  * FQSL_ERR_ARG (NULL, or no timed call yet), FQSL_ERR_CUDA. */
 FQSL_API fqsl_status fqsl_field_set_timing(fqsl_field field, int enable);
 FQSL_API fqsl_status fqsl_field_times(fqsl_field field, float ms[3]);
@@ -296,8 +298,9 @@ FQSL_API fqsl_status fqsl_batch_create(const fqsl_field *fields, const fqsl_plan
 
 /* Run a batch plan on cuda_stream: one seed pre-pass (FP32), one persistent
  * tracer launch over the work items of all entries (a device counter hands
- * out 8x4-seed tiles of any entry), one launch for the rotated-S0 extra lines
- * of all entries (if any plane is interior) and one assembly launch. No
+ * out 8x4-seed tiles of any entry, and after them the rotated-S0 extra lines of
+ * the entries whose plane is interior; FP64: those in a second launch) and one
+ * assembly launch. No
  * allocation and no host synchronisation happen here. */
 FQSL_API fqsl_status fqsl_batch_run(fqsl_batch batch, void *cuda_stream);
 

@@ -586,10 +586,105 @@ DevParams dev_params(const fqsl_params *p)
     d.scheme = p->scheme;
     d.step = p->step;
     d.step_min = p->step_min;
+    d.lanes = 32;
+    d.split = 0;
+    d.merge = 0;
     return d;
 }
 
+// How an untaped launch spreads its lines over the GPU.
+struct Spread {
+    int bps;     // resident 128-thread blocks per SM
+    int lanes;   // lanes of a warp that take lines
+    bool split;  // the two directions of a line as separate items (FP32)
+};
+
+// What kind of seeds a launch has.
+enum SeedKind {
+    kSeedsFace,    // a lattice on a face of the box: one direction of each line ends at once
+    kSeedsInside,  // a lattice inside the box
+    kSeedsList     // an explicit list: neighbours in it need not be neighbours in space
+};
+
+// Blocks per SM. FP32 lines that share no cells (lists; lattices at least a
+// cell apart) touch pages of the node records all over a large cube, and more
+// resident lanes than the address translation can serve make each load slower
+// than they hide: nothing but the latency is busy (ncu, 2.1 GB of records, 4
+// blocks: L1 24 %, L2 19 %, DRAM 25 %; 2 blocks are 1.4 times as fast with the
+// same DRAM traffic). Measured on GB300, ms at 4 / 3 / 2 blocks:
+//   records   lattice of 96x96x48 seeds      list of 300,000 seeds
+//   0.27 GB   4.38 /  4.64 /  5.66          2.49 /  2.86 /  3.55
+//   0.52 GB   5.58 /  5.98 /  7.38          4.46 /  3.72 /  4.56
+//   0.91 GB   7.76 /  7.44 /  9.02          7.41 /  6.48 /  5.71
+//   1.44 GB  14.22 /  9.20 / 10.70          9.96 /  8.67 /  7.17
+//   2.15 GB  20.01 / 11.83 / 12.49         12.19 / 10.58 /  8.53
+// (a plane of 1024x512 seeds half a cell apart in the last cube: 5.43 / 5.86 / 7.40)
+int tlb_blocks(size_t record_bytes, SeedKind kind, bool sparse, int bps)
+{
+    if (!sparse) return bps;
+    int most = bps;
+    if (kind == kSeedsList) most = record_bytes >= ((size_t)700 << 20) ? 2 : (record_bytes >= ((size_t)400 << 20) ? 3 : bps);
+    else if (record_bytes >= ((size_t)1200 << 20)) most = 3;
+    return most < bps ? most : bps;
+}
+
+// Spread `lines` lines over the GPU.
+//   split: a lattice inside the box up to three times the resident lanes (a
+//     launch that small ends on its longest lines: 16,384 seeds of a vertical
+//     cut of a 256x256x128 cube 0.75 -> 0.51 ms, 202,500 1.65 -> 1.58 ms; a
+//     volume of 131,072 with the fixed step 6.07 -> 4.52 ms; Method II, whose
+//     lines are heavier, only while all directions are resident: 54,600 seeds
+//     of a 88x66x50 cube 0.57 -> 0.66 ms), and a list so
+//     short that every direction gets a warp of its own (a longer list gains
+//     nothing: 8,000 seeds 0.456 ms either way, 30,000 0.61 against 0.54 ms).
+//     Not a lattice on a box face, where one direction ends at once and its
+//     lanes would idle (90,000 seeds 0.62 -> 1.17 ms).
+//   lanes: fewer lines per warp until the lines fill the resident warps: lanes
+//     of one warp whose lines have parted wait for each other's loads (list of
+//     500 seeds 0.36 -> 0.26 ms with 2 lanes, plane of 4,096 seeds 0.38 -> 0.32
+//     ms with 4, of 40,000 0.58 -> 0.51 ms with 16; with more warps than fit at
+//     once it loses: 90,000 seeds of a plane 0.62 -> 0.84 ms, a list of 40,604
+//     seeds 0.45 -> 0.56 ms). FP64 warp instructions
+//     take the narrow FP64 pipe the same time whatever their lanes, so FP64
+//     lines are spread only over SMs that would idle.
+Spread spread_of(const fqsl_field f, const fqsl_params *p, int bps, long long lines, SeedKind kind, bool sparse,
+                 bool may_split)
+{
+    const bool f32 = p->precision != FQSL_F64;
+    Spread r{bps, 32, false};
+    if (p->blocks_per_sm > 0) r.bps = p->blocks_per_sm < bps ? p->blocks_per_sm : bps;
+    else if (f32 && lines > (long long)f->sms * kTraceBlock) r.bps = tlb_blocks((size_t)f->g.nodes * 32, kind, sparse, bps);
+    const long long warps = (long long)f->sms * r.bps * (kTraceBlock / 32);
+    if (f32 && may_split && kind == kSeedsInside) r.split = lines <= (p->method == 2 ? 16 : 96) * warps;
+    if (f32 && may_split && kind == kSeedsList) r.split = 2 * lines <= warps;
+    const long long items = (r.split ? 2 : 1) * lines;
+    const long long most = !f32 ? f->sms : (kind == kSeedsFace ? warps + warps / 16 : warps);
+    if (p->chunk_tiles == 0)
+        while (r.lanes > 1 && items <= most * (r.lanes / 2)) r.lanes /= 2;
+    return r;
+}
+
+// Are a lattice's seeds a cell or more apart (its 8x4-seed tile covers at
+// least as many cells as it has seeds)?
+bool sparse_lattice(const FieldView &g, const Lattice &lat)
+{
+    double area = 1.0;
+    const double *step[2] = {lat.a1, lat.a2};
+    const int n[3] = {g.nx, g.ny, g.nz};
+    for (int q = 0; q < 2; q++) {
+        double s = 0.0;
+        for (int a = 0; a < 3; a++) {
+            const double d = g.rect ? (g.hi64[a] - g.lo64[a]) / (n[a] - 1) : g.d[a];
+            s = fmax(s, fabs(step[q][a]) / d);
+        }
+        area *= s;
+    }
+    return area >= 1.0;
+}
+
 struct Scratch {
+    unsigned long long *ctr = nullptr;  // [0], [1] work counters, [2] rotated seeds (low 32 bits)
+    size_t zero_bytes = 0;              // from ctr on: cleared before the launch (counters, pair, rot_slot)
     LineRecs rec{}, ext{};
     SeedPrep prep{};
     int32_t *rot_seed = nullptr, *rot_slot = nullptr;
@@ -597,14 +692,20 @@ struct Scratch {
 };
 
 // Lay out the per-call scratch for n primary lines (and 4 n extra lines when
-// rotation is possible): FP64 records for the FP64 tracer, index-space
-// records and the seed pre-pass arrays for the FP32 tracers. With base == NULL
-// only the size is computed.
-Scratch layout(char *base, long long n, bool rot, bool lattice, bool f32, bool m2 = false)
+// rotation is possible, their records behind the primary lines'): FP64 records
+// for the FP64 tracer, index-space records and the seed pre-pass arrays for the
+// FP32 tracers; pair: also the words of split directions. With base == NULL only
+// the size is computed.
+Scratch layout(char *base, long long n, bool rot, bool lattice, bool f32, bool m2 = false, bool pair = false)
 {
     Carver c{base};
     Scratch s;
     LineRecs &r = s.rec;
+    const long long m = rot ? 5 * n : n;
+    s.ctr = c.take<unsigned long long>(4);
+    if (pair) r.pair = c.take<unsigned long long>(m);
+    if (rot) s.rot_slot = c.take<int32_t>(n);
+    s.zero_bytes = c.off;
     if (m2) {
         if (f32) {
             r.dev32 = c.take<float>(12 * n);
@@ -616,41 +717,40 @@ Scratch layout(char *base, long long n, bool rot, bool lattice, bool f32, bool m
         }
     }
     if (f32) {
-        r.xi1 = c.take<float>(3 * n);
-        r.xi2 = c.take<float>(3 * n);
+        r.xi1 = c.take<float>(3 * m);
+        r.xi2 = c.take<float>(3 * m);
         r.kacc = c.take<float4>(2 * n);
     } else {
-        r.r1 = c.take<double>(3 * n);
-        r.r2 = c.take<double>(3 * n);
+        r.r1 = c.take<double>(3 * m);
+        r.r2 = c.take<double>(3 * m);
         r.bn1 = lattice ? c.take<double>(n) : nullptr;
         r.bn2 = lattice ? c.take<double>(n) : nullptr;
         r.tw = c.take<double>(n);
         r.len = c.take<double>(n);
     }
     r.bn0 = lattice ? c.take<double>(n) : nullptr;
-    r.f1 = c.take<int8_t>(n);
-    r.f2 = c.take<int8_t>(n);
-    r.st = c.take<uint8_t>(n);
-    r.steps = c.take<int32_t>(n);
+    r.f1 = c.take<int8_t>(m);
+    r.f2 = c.take<int8_t>(m);
+    r.st = c.take<uint8_t>(m);
+    r.steps = c.take<int32_t>(m);
     if (f32 && lattice) {
         s.prep.seed = c.take<float4>(n);
         s.prep.flags = c.take<uint8_t>(n);
     }
     if (rot) {
         s.rot_seed = c.take<int32_t>(n);
-        s.rot_slot = c.take<int32_t>(n);
         LineRecs &x = s.ext;
         if (f32) {
-            x.xi1 = c.take<float>(12 * n);
-            x.xi2 = c.take<float>(12 * n);
+            x.xi1 = r.xi1 + 3 * n;
+            x.xi2 = r.xi2 + 3 * n;
         } else {
-            x.r1 = c.take<double>(12 * n);
-            x.r2 = c.take<double>(12 * n);
+            x.r1 = r.r1 + 3 * n;
+            x.r2 = r.r2 + 3 * n;
         }
-        x.f1 = c.take<int8_t>(4 * n);
-        x.f2 = c.take<int8_t>(4 * n);
-        x.st = c.take<uint8_t>(4 * n);
-        x.steps = c.take<int32_t>(4 * n);
+        x.f1 = r.f1 + n;
+        x.f2 = r.f2 + n;
+        x.st = r.st + n;
+        x.steps = r.steps + n;
     }
     s.bytes = c.off;
     return s;
@@ -693,22 +793,47 @@ int blocks_per_sm(fqsl_field f, int precision, int src, int p_scheme)
     return c;
 }
 
-cudaError_t launch_trace(fqsl_field f, const fqsl_params *p, const TraceArgs &a, int src, long long items,
-                         cudaStream_t s)
+// The grid of a launch of `items` items spread as sp says; full: lines that the
+// host cannot count follow (extra lines), so the grid fills the GPU.
+long long spread_grid(const Spread &sp, int sms, long long items, bool full)
 {
-    const long long warps_needed = (items + 31) / 32;
-    int bps = blocks_per_sm(f, p->precision, src, p->scheme);
-    if (p->blocks_per_sm > 0 && p->blocks_per_sm < bps) bps = p->blocks_per_sm;
-    long long grid = (long long)f->sms * bps;
-    const long long need = (warps_needed * 32 + kTraceBlock - 1) / kTraceBlock;
-    if (src != kSrcExtra && need < grid) grid = need;
-    if (grid < 1) grid = 1;
+    long long grid = (long long)sms * sp.bps;
+    const long long per_block = (long long)sp.lanes * (kTraceBlock / 32);
+    const long long need = ((sp.split ? 2 : 1) * items + per_block - 1) / per_block;
+    if (!full && need < grid) grid = need;
+    return grid < 1 ? 1 : grid;
+}
+
+void set_spread(TraceArgs &a, const Spread &sp)
+{
+    a.p.lanes = sp.lanes;
+    a.p.split = sp.split ? 1 : 0;
+    if (sp.lanes < 32) a.p.chunk = sp.lanes;
+    else if (sp.split) a.p.chunk = kTileU * kTileV;
+}
+
+cudaError_t launch_trace(const fqsl_params *p, const TraceArgs &a, int src, long long grid, cudaStream_t s)
+{
     return p->precision == FQSL_F64 ? launch_trace_f64(a, src, (int)grid, kTraceBlock, s)
                                     : launch_trace_f32(a, src, (int)grid, kTraceBlock, s,
                                                        p->precision == FQSL_F32_ACC64);
 }
 
-cudaError_t launch_trace_m2(fqsl_field f, const fqsl_params *p, const TraceArgs &a, cudaStream_t s)
+// The extra lines of rotated seeds in a launch of their own: the FP32 lattice
+// kernel with no lattice items, the FP64 one's own source.
+cudaError_t launch_extra(fqsl_field f, const fqsl_params *p, TraceArgs a, const Scratch &s, const Spread &sp,
+                         cudaStream_t stream)
+{
+    a.q.head = s.ctr + 1;
+    const bool f32 = p->precision != FQSL_F64;
+    if (f32) {
+        a.nitems = 0;
+        a.p.merge = 1;
+    }
+    return launch_trace(p, a, f32 ? kSrcLattice : kSrcExtra, spread_grid(sp, f->sms, 0, true), stream);
+}
+
+int blocks_per_sm_m2(fqsl_field f, const fqsl_params *p)
 {
     int &c = f->blocks_cache_m2[p->scheme][p->precision == FQSL_F64 ? 1 : 0][p->gradb_way - 1];
     if (!c) {
@@ -725,10 +850,11 @@ cudaError_t launch_trace_m2(fqsl_field f, const fqsl_params *p, const TraceArgs 
             c = p->precision == FQSL_F64 ? trace_dev_blocks_per_sm_f64(p->gradb_way)
                                          : trace_dev_blocks_per_sm_f32(p->gradb_way);
     }
-    long long grid = (long long)f->sms * (p->blocks_per_sm > 0 && p->blocks_per_sm < c ? p->blocks_per_sm : c);
-    const long long need = (a.nitems + kTraceBlock - 1) / kTraceBlock;
-    if (need < grid) grid = need;
-    if (grid < 1) grid = 1;
+    return c;
+}
+
+cudaError_t launch_trace_m2(const fqsl_params *p, const TraceArgs &a, long long grid, cudaStream_t s)
+{
     return p->precision == FQSL_F64 ? launch_trace_dev_f64(a, p->gradb_way, (int)grid, kTraceBlock, s)
                                     : launch_trace_dev_f32(a, p->gradb_way, (int)grid, kTraceBlock, s);
 }
@@ -906,8 +1032,13 @@ fqsl_status run_qmap_locked(fqsl_field f, const Lattice &lat0, const fqsl_params
     lat.allow_rot = (p->method == 1 && !face_plane) ? 1 : 0;
     const bool f32 = p->precision != FQSL_F64;
     const bool m2 = p->method == 2;
+    const bool rot = lat.allow_rot != 0;
     Scratch s;
+    Spread sp{};
     TapeLayout tl{};
+    if (!tape)
+        sp = spread_of(f, p, m2 ? blocks_per_sm_m2(f, p) : blocks_per_sm(f, p->precision, kSrcLattice, p->scheme), n,
+                       face_plane ? kSeedsFace : kSeedsInside, sparse_lattice(f->g, lat), true);
     if (tape) {
         tape->valid = false;
         tape->field = f;
@@ -930,14 +1061,13 @@ fqsl_status run_qmap_locked(fqsl_field f, const Lattice &lat0, const fqsl_params
         tl = tape_layout_of(tape, (char *)tape->buf, tape->pool);
         s = tl.s;
     } else {
-        Scratch sz = layout(nullptr, n, lat.allow_rot, true, f32, m2);
+        Scratch sz = layout(nullptr, n, rot, true, f32, m2, sp.split);
         fqsl_status st = ensure_scratch(f, sz.bytes);
         if (st != FQSL_OK) return st;
-        s = layout((char *)f->scratch, n, lat.allow_rot, true, f32, m2);
+        s = layout((char *)f->scratch, n, rot, true, f32, m2, sp.split);
     }
 
-    cudaError_t e = cudaMemsetAsync(f->counters, 0, 4 * sizeof(unsigned long long), stream);
-    if (e == cudaSuccess && lat.allow_rot) e = cudaMemsetAsync(s.rot_slot, 0, (size_t)n * sizeof(int32_t), stream);
+    cudaError_t e = cudaMemsetAsync(s.ctr, 0, s.zero_bytes, stream);
     if (e == cudaSuccess && tape) e = cudaMemsetAsync(tl.ctr, 0, 6 * sizeof(unsigned long long), stream);
     if (e == cudaSuccess && tape) {
         // the taped tracer traces the two directions of a line as separate
@@ -957,22 +1087,24 @@ fqsl_status run_qmap_locked(fqsl_field f, const Lattice &lat0, const fqsl_params
     a.lat = lat;
     a.rec = s.rec;
     a.ext = s.ext;
-    a.q.head = f->counters;
-    // a taped map keeps its rotated-seed count with the tape (f->counters is
-    // shared with the field's other calls)
-    a.q.rot_count = tape ? (unsigned int *)(tl.ctr + 4) : (unsigned int *)(f->counters + 2);
+    a.q.head = s.ctr;
+    // a taped map keeps its rotated-seed count with the tape
+    a.q.rot_count = tape ? (unsigned int *)(tl.ctr + 4) : (unsigned int *)(s.ctr + 2);
     a.q.rot_seed = s.rot_seed;
     a.q.rot_slot = s.rot_slot;
     a.prep = s.prep;
     a.tape = tl.tape;
     a.nitems = lat.n3 * lat.tiles_u * lat.tiles_v * (long long)(kTileU * kTileV);
+    if (!tape) set_spread(a, sp);
+    // (with timing on, the extra lines get a launch of their own to be timed)
+    a.p.merge = !tape && f32 && rot && !f->timing;
     if (f32) {
         e = launch_seed_prep_f32(a, n, stream);
         if (e != cudaSuccess) return cuda_fail(e, who);
     }
     mark(f, 0, stream);
     if (m2) {
-        e = launch_trace_m2(f, p, a, stream);
+        e = launch_trace_m2(p, a, spread_grid(sp, f->sms, a.nitems, false), stream);
         if (e != cudaSuccess) return cuda_fail(e, who);
         mark(f, 1, stream);
         mark(f, 2, stream);
@@ -1001,11 +1133,11 @@ fqsl_status run_qmap_locked(fqsl_field f, const Lattice &lat0, const fqsl_params
         if (grid < 1) grid = 1;
         e = launch_tape(a, p, kSrcLattice, grid, stream);
     } else {
-        e = launch_trace(f, p, a, kSrcLattice, a.nitems, stream);
+        e = launch_trace(p, a, kSrcLattice, spread_grid(sp, f->sms, a.nitems, a.p.merge != 0), stream);
     }
     if (e != cudaSuccess) return cuda_fail(e, who);
     mark(f, 1, stream);
-    if (lat.allow_rot) {
+    if (rot && !a.p.merge) {
         if (tape) {
             // the extra lines' half-lines follow the lattice's on the tape;
             // their count is read on the device (persistent grid)
@@ -1015,8 +1147,7 @@ fqsl_status run_qmap_locked(fqsl_field f, const Lattice &lat0, const fqsl_params
             if (p->blocks_per_sm > 0 && p->blocks_per_sm < bps) bps = p->blocks_per_sm;
             e = launch_tape(a, p, kSrcExtra, (long long)f->sms * bps, stream);
         } else {
-            a.q.head = f->counters + 1;
-            e = launch_trace(f, p, a, kSrcExtra, 4 * n, stream);
+            e = launch_extra(f, p, a, s, sp, stream);
         }
         if (e != cudaSuccess) return cuda_fail(e, who);
     }
@@ -1054,7 +1185,7 @@ fqsl_status run_qmap_locked(fqsl_field f, const Lattice &lat0, const fqsl_params
     if (e != cudaSuccess) return cuda_fail(e, who);
     mark(f, 3, stream);
     f->timed = f->timing;
-    f->extra_timed = lat.allow_rot != 0;
+    f->extra_timed = rot;
     if (tape) tape->valid = true;
     return FQSL_OK;
 }
@@ -1203,11 +1334,12 @@ fqsl_status fqsl_twist(fqsl_field f, const double *seeds_dev, long long n, const
     cudaStream_t stream = (cudaStream_t)cuda_stream;
     const bool f32 = p->precision != FQSL_F64;
     std::lock_guard<std::mutex> lock(f->mu);
-    Scratch sz = layout(nullptr, n, false, false, f32);
+    const Spread sp = spread_of(f, p, blocks_per_sm(f, p->precision, kSrcList, p->scheme), n, kSeedsList, true, true);
+    Scratch sz = layout(nullptr, n, false, false, f32, false, sp.split);
     st = ensure_scratch(f, sz.bytes);
     if (st != FQSL_OK) return st;
-    Scratch s = layout((char *)f->scratch, n, false, false, f32);
-    cudaError_t e = cudaMemsetAsync(f->counters, 0, 4 * sizeof(unsigned long long), stream);
+    Scratch s = layout((char *)f->scratch, n, false, false, f32, false, sp.split);
+    cudaError_t e = cudaMemsetAsync(s.ctr, 0, s.zero_bytes, stream);
     if (e != cudaSuccess) return cuda_fail(e, who);
     TraceArgs a{};
     a.f = f->g;
@@ -1216,9 +1348,10 @@ fqsl_status fqsl_twist(fqsl_field f, const double *seeds_dev, long long n, const
     a.seeds = seeds_dev;
     a.nitems = n;
     a.rec = s.rec;
-    a.q.head = f->counters;
+    a.q.head = s.ctr;
+    set_spread(a, sp);
     mark(f, 0, stream);
-    e = launch_trace(f, p, a, kSrcList, n, stream);
+    e = launch_trace(p, a, kSrcList, spread_grid(sp, f->sms, (n + 31) / 32 * 32, false), stream);
     if (e != cudaSuccess) return cuda_fail(e, who);
     mark(f, 1, stream);
     mark(f, 2, stream);
@@ -1334,20 +1467,25 @@ extern "C" fqsl_status fqsl_qmap_plane_static(fqsl_field f, const double origin[
     char *base = nullptr;
     st = static_scratch(&base);
     if (st != FQSL_OK) return st;
-    // counters first, then the line records
-    unsigned long long *counters = (unsigned long long *)base;
-    const size_t head = 256;
     const bool f32 = p->precision != FQSL_F64;
-    Scratch need = layout(nullptr, n, lat.allow_rot, true, f32);
-    if (head + need.bytes > kStaticScratchBytes)
+    const bool rot = lat.allow_rot != 0;
+    std::lock_guard<std::mutex> lock(f->mu);
+    const SeedKind kind = face_plane ? kSeedsFace : kSeedsInside;
+    const bool sparse = sparse_lattice(f->g, lat);
+    const int bps = blocks_per_sm(f, p->precision, kSrcLattice, p->scheme);
+    Spread sp = spread_of(f, p, bps, n, kind, sparse, true);
+    Scratch need = layout(nullptr, n, rot, true, f32, false, sp.split);
+    if (need.bytes > kStaticScratchBytes && sp.split) {
+        sp = spread_of(f, p, bps, n, kind, sparse, false);
+        need = layout(nullptr, n, rot, true, f32);
+    }
+    if (need.bytes > kStaticScratchBytes)
         return fail(FQSL_ERR_ARG, "%s: %lld seeds need %zu scratch bytes, the static array holds %zu", who, n,
-                    head + need.bytes, kStaticScratchBytes);
-    Scratch s = layout(base + head, n, lat.allow_rot, true, f32);
+                    need.bytes, kStaticScratchBytes);
+    Scratch s = layout(base, n, rot, true, f32, false, sp.split);
     cudaStream_t stream = (cudaStream_t)cuda_stream;
 
-    std::lock_guard<std::mutex> lock(f->mu);
-    cudaError_t e = cudaMemsetAsync(counters, 0, 4 * sizeof(unsigned long long), stream);
-    if (e == cudaSuccess && lat.allow_rot) e = cudaMemsetAsync(s.rot_slot, 0, (size_t)n * sizeof(int32_t), stream);
+    cudaError_t e = cudaMemsetAsync(s.ctr, 0, s.zero_bytes, stream);
     if (e != cudaSuccess) return cuda_fail(e, who);
     TraceArgs a{};
     a.f = f->g;
@@ -1356,23 +1494,24 @@ extern "C" fqsl_status fqsl_qmap_plane_static(fqsl_field f, const double origin[
     a.lat = lat;
     a.rec = s.rec;
     a.ext = s.ext;
-    a.q.head = counters;
-    a.q.rot_count = (unsigned int *)(counters + 2);
+    a.q.head = s.ctr;
+    a.q.rot_count = (unsigned int *)(s.ctr + 2);
     a.q.rot_seed = s.rot_seed;
     a.q.rot_slot = s.rot_slot;
     a.prep = s.prep;
     a.nitems = lat.n3 * lat.tiles_u * lat.tiles_v * (long long)(kTileU * kTileV);
+    set_spread(a, sp);
+    a.p.merge = f32 && rot && !f->timing;
     if (f32) {
         e = launch_seed_prep_f32(a, n, stream);
         if (e != cudaSuccess) return cuda_fail(e, who);
     }
     mark(f, 0, stream);
-    e = launch_trace(f, p, a, kSrcLattice, a.nitems, stream);
+    e = launch_trace(p, a, kSrcLattice, spread_grid(sp, f->sms, a.nitems, a.p.merge != 0), stream);
     if (e != cudaSuccess) return cuda_fail(e, who);
     mark(f, 1, stream);
-    if (lat.allow_rot) {
-        a.q.head = counters + 1;
-        e = launch_trace(f, p, a, kSrcExtra, 4 * n, stream);
+    if (rot && !a.p.merge) {
+        e = launch_extra(f, p, a, s, sp, stream);
         if (e != cudaSuccess) return cuda_fail(e, who);
     }
     mark(f, 2, stream);
@@ -1389,7 +1528,7 @@ extern "C" fqsl_status fqsl_qmap_plane_static(fqsl_field f, const double origin[
     if (e != cudaSuccess) return cuda_fail(e, who);
     mark(f, 3, stream);
     f->timed = f->timing;
-    f->extra_timed = lat.allow_rot != 0;
+    f->extra_timed = rot;
     return FQSL_OK;
 }
 
@@ -1613,20 +1752,24 @@ extern "C" fqsl_status fqsl_batch_run(fqsl_batch b, void *cuda_stream)
     a0.p.chunk = kTileU * kTileV;  // a grab never spans two entries
     a0.q.head = b->d_heads;
     a0.nitems = b->total_items;
-    BatchArgs ba{b->d_desc, b->d_ibase, b->nent};
+    a0.p.merge = f32 && b->any_rot;
+    if (a0.p.merge) {
+        e = launch_batch_extra_prefix(b->d_rot_counts, b->nent, b->d_xbase, s);
+        if (e != cudaSuccess) return cuda_fail(e, who);
+    }
+    BatchArgs ba{b->d_desc, b->d_ibase, b->nent, b->d_xbase};
     long long grid = b->grid;
     const long long need = (b->total_items + kTraceBlock - 1) / kTraceBlock;
-    if (need < grid) grid = need;
-    e = f32 ? launch_batch_trace_f32(a0, ba, kSrcLattice, p->precision == FQSL_F32_ACC64, (int)grid, s)
+    if (!a0.p.merge && need < grid) grid = need;
+    e = f32 ? launch_batch_trace_f32(a0, ba, p->precision == FQSL_F32_ACC64, (int)grid, s)
             : launch_batch_trace_f64(a0, ba, kSrcLattice, (int)grid, s);
     if (e != cudaSuccess) return cuda_fail(e, who);
-    if (b->any_rot) {
+    if (b->any_rot && !a0.p.merge) {
         e = launch_batch_extra_prefix(b->d_rot_counts, b->nent, b->d_xbase, s);
         if (e != cudaSuccess) return cuda_fail(e, who);
         a0.q.head = b->d_heads + 1;
-        BatchArgs bx{b->d_desc, b->d_xbase, b->nent};
-        e = f32 ? launch_batch_trace_f32(a0, bx, kSrcExtra, p->precision == FQSL_F32_ACC64, b->grid, s)
-                : launch_batch_trace_f64(a0, bx, kSrcExtra, b->grid, s);
+        BatchArgs bx{b->d_desc, b->d_xbase, b->nent, nullptr};
+        e = launch_batch_trace_f64(a0, bx, kSrcExtra, b->grid, s);
         if (e != cudaSuccess) return cuda_fail(e, who);
     }
     e = f32 ? launch_batch_assemble_f32(b->d_adesc, b->d_nbase, b->nent, b->total_seeds, s)

@@ -69,7 +69,10 @@ struct DevParams {
     int method, way;
     int refill;     // minimum idle lanes before a warp takes new seeds
     int sync_dirs;  // lanes wait for each other before their second direction
-    int chunk;      // work items per grab of the counter (a multiple of 32)
+    int chunk;      // work items per grab of the counter (a multiple of 32, or lanes where lanes < 32)
+    int lanes;      // lanes of a warp that take lines (a power of two, at most 32)
+    int split;      // FP32: the two directions of a line are separate items (LineRecs::pair)
+    int merge;      // FP32 lattices: the rotated seeds' extra lines follow the lattice's items
     int scheme;     // 0 = RKF45, 1 = fixed-step 3/8 rule
     double step, step_min;  // fixed-step scheme: step_perp and Eq. step's floor (cells)
 };
@@ -112,6 +115,7 @@ struct LineRecs {
     int8_t *f1, *f2;
     uint8_t *st;
     int32_t *steps;
+    unsigned long long *pair;  // DevParams::split: one word per line, zero before the launch
 };
 
 // FP32 seed pre-pass output: index-space seed and tol^2, and flags.
@@ -194,6 +198,7 @@ struct BatchArgs {
     const TraceArgs *desc;  // per entry (device memory)
     const long long *ibase;
     int nent;
+    const long long *xbase;  // the same for the rotated seeds' extra lines (DevParams::merge)
 };
 
 struct AssembleArgs {
@@ -327,13 +332,13 @@ cudaError_t launch_seed_prep_f32(const TraceArgs &a, long long n, cudaStream_t s
 cudaError_t launch_batch_seed_prep_f32(const TraceArgs *desc, const long long *nbase, int nent, long long total,
                                        cudaStream_t s);
 cudaError_t launch_batch_extra_prefix(const unsigned *rot_counts, int nent, long long *xbase, cudaStream_t s);
-cudaError_t launch_batch_trace_f32(const TraceArgs &a0, const BatchArgs &b, int src, bool acc64, int grid,
+cudaError_t launch_batch_trace_f32(const TraceArgs &a0, const BatchArgs &b, bool acc64, int grid,
                                    cudaStream_t s);
 cudaError_t launch_batch_trace_f64(const TraceArgs &a0, const BatchArgs &b, int src, int grid, cudaStream_t s);
 int batch_trace_blocks_per_sm_f32(bool acc64, int scheme);
 int batch_trace_blocks_per_sm_f64(int scheme);
 // the same with the fixed-step scheme (trace_rk38_f32.cu, trace_rk38_f64.cu)
-cudaError_t launch_batch_trace_rk38_f32(const TraceArgs &a0, const BatchArgs &b, int src, bool acc64, int grid,
+cudaError_t launch_batch_trace_rk38_f32(const TraceArgs &a0, const BatchArgs &b, bool acc64, int grid,
                                         cudaStream_t s);
 cudaError_t launch_batch_trace_rk38_f64(const TraceArgs &a0, const BatchArgs &b, int src, int grid, cudaStream_t s);
 int batch_trace_rk38_blocks_per_sm_f32(bool acc64);

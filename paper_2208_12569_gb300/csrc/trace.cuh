@@ -938,6 +938,11 @@ struct Lane {
     T u[3], v[3], u0[3], v0[3], ou[3], ov[3];
 };
 
+// Lane::st holds the line's status bits in its low byte and, above them, how the
+// lane came by the line.
+constexpr int kLaneExtra = 0x100;  // an extra line of a rotated seed (no length/Tw sums are kept)
+constexpr int kLaneSplit = 0x200;  // the line's other direction is another lane's (see split_join)
+
 // Length and Tw of the current direction: FP64 sums (ACC, and the FP64
 // tracer) or compensated FP32 sums (Kahan 1965) whose total is formed in FP64
 // once per direction.
@@ -1133,10 +1138,71 @@ __device__ __forceinline__ void split_finish(const TraceArgs &A, const LineRecs 
     }
 }
 
+// Start the second direction of a line at its seed.
+template <typename T, bool ACC, int DEV = 0>
+__device__ __forceinline__ void start_second(const TraceArgs &A, Lane<T> &L)
+{
+    L.end = 1;
+    L.x = L.sx;
+    L.y = L.sy;
+    L.z = L.sz;
+    if constexpr (DEV != 0) {
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            L.u[c] = L.u0[c];
+            L.v[c] = L.v0[c];
+        }
+    }
+    L.h = A.p.scheme == 1 ? (T)L.tol : (T)A.p.h0;  // fixed step: the line's step (in tol)
+    L.mode = 0;
+    L.tcur = -1;
+    L.tn = 0;
+    acc_reset<T, ACC>(L);
+}
+
+// Untaped maps too small to fill the GPU give the two directions of a line to
+// two lanes (kLaneSplit; FP32). Each lane adds its trial count (bits 0-31), its
+// status (bits 32-39 and 40-47) and how it ended (48, 49: done; 50, 51: bad)
+// to the line's pair word, and the lane that comes second writes the line's
+// record as one lane tracing both directions would have: a bad first direction
+// ends the line (end 2 is the seed, only the first direction's trials count),
+// and if both together reach max_steps the second direction is traced again
+// with what the first left of the budget. Returns whether this lane has to.
+template <typename T, bool ACC, int DEV>
+__device__ __forceinline__ bool split_join(const TraceArgs &A, const LineRecs &R, Lane<T> &L, bool bad)
+{
+    if (L.end == 0) *(volatile int32_t *)(R.steps + L.line) = L.steps;
+    const unsigned long long mine = (unsigned long long)(unsigned)L.steps |
+                                    ((unsigned long long)((unsigned)L.st & 0xffu) << (32 + 8 * L.end)) |
+                                    (1ull << (48 + L.end)) | ((bad ? 1ull : 0ull) << (50 + L.end));
+    __threadfence();  // this direction's end record, before the other lane can see it as done
+    const unsigned long long old = atomicAdd(R.pair + L.line, mine);
+    if (((old >> 48) & 3ull) == 0ull) return false;
+    __threadfence();
+    const unsigned long long both = old + mine;
+    const unsigned st0 = (unsigned)(both >> 32) & 0xffu, st1 = (unsigned)(both >> 40) & 0xffu;
+    const int32_t steps0 = *(volatile int32_t *)(R.steps + L.line);
+    if ((both >> 50) & 1ull) {
+        write_end32(R, L.line, 1, (float)L.sx, (float)L.sy, (float)L.sz, -1);
+        R.st[L.line] = (uint8_t)st0;
+        return false;
+    }
+    if ((both & 0xffffffffull) >= (unsigned long long)A.p.max_steps) {
+        L.st = (int)st0 | (L.st & kLaneExtra);
+        L.steps = steps0;
+        start_second<T, ACC, DEV>(A, L);
+        return true;
+    }
+    R.st[L.line] = (uint8_t)(st0 | st1);
+    R.steps[L.line] = (int32_t)(both & 0xffffffffull);
+    return false;
+}
+
 // Finish the line with a bad status (MAXSTEPS or NULL_B): the unfinished end
 // is the current position, an untraced end the seed, their faces -1.
-template <typename T, bool SPLIT = false, bool RECT = false>
-__device__ __forceinline__ void finish_bad(const TraceArgs &A, const LineRecs &R, Lane<T> &L, unsigned bit)
+// Returns whether the lane goes on with the line (split_join).
+template <typename T, bool ACC, int DEV = 0, bool SPLIT = false, bool RECT = false, bool FLEX = false>
+__device__ __forceinline__ bool finish_bad(const TraceArgs &A, const LineRecs &R, Lane<T> &L, unsigned bit)
 {
     const FieldView &f = A.f;
     L.st |= bit;
@@ -1150,7 +1216,11 @@ __device__ __forceinline__ void finish_bad(const TraceArgs &A, const LineRecs &R
         if (R.len) R.len[L.line] = NAN;
     } else {
         write_end32(R, L.line, L.end, (float)L.x, (float)L.y, (float)L.z, -1);
-        if (L.end == 0 && !SPLIT) write_end32(R, L.line, 1, (float)L.sx, (float)L.sy, (float)L.sz, -1);
+        if constexpr (!SPLIT) {
+            if constexpr (FLEX)
+                if (L.st & kLaneSplit) return split_join<T, ACC, DEV>(A, R, L, true);
+            if (L.end == 0) write_end32(R, L.line, 1, (float)L.sx, (float)L.sy, (float)L.sz, -1);
+        }
     }
     if constexpr (SPLIT) {
         split_finish(A, R, L, true);
@@ -1158,11 +1228,12 @@ __device__ __forceinline__ void finish_bad(const TraceArgs &A, const LineRecs &R
         R.st[L.line] = (uint8_t)L.st;
         R.steps[L.line] = L.steps;
     }
+    return false;
 }
 
 // A direction reached a face at index position (x, y, z) with deviation
 // vectors (du, dv) (Method II only).
-template <typename T, bool ACC, int DEV = 0, bool SPLIT = false, bool RECT = false>
+template <typename T, bool ACC, int DEV = 0, bool SPLIT = false, bool RECT = false, bool FLEX = false>
 __device__ __forceinline__ bool finish_dir(const TraceArgs &A, const LineRecs &R, Lane<T> &L, T x, T y, T z,
                                            int face, const T *du = nullptr, const T *dv = nullptr)
 {
@@ -1198,7 +1269,7 @@ __device__ __forceinline__ bool finish_dir(const TraceArgs &A, const LineRecs &R
         }
     } else {
         write_end32(R, L.line, L.end, (float)x, (float)y, (float)z, face);
-        if (R.kacc) {
+        if (R.kacc && !(FLEX && (L.st & kLaneExtra))) {
             float4 k;
             if (ACC) {
                 // FP64 sums: carry the value and its float residue
@@ -1218,27 +1289,15 @@ __device__ __forceinline__ bool finish_dir(const TraceArgs &A, const LineRecs &R
         split_finish(A, R, L, false);
         return false;
     }
+    if constexpr (FLEX) {
+        if (L.st & kLaneSplit) return split_join<T, ACC, DEV>(A, R, L, false);
+    }
     if (L.end == 0) {
         if constexpr (sizeof(T) == 8) {
             L.l1 = acc_len<T, ACC>(L);
             L.tw1 = acc_tw<T, ACC>(L);
         }
-        L.end = 1;
-        L.x = L.sx;
-        L.y = L.sy;
-        L.z = L.sz;
-        if constexpr (DEV != 0) {
-#pragma unroll
-            for (int c = 0; c < 3; c++) {
-                L.u[c] = L.u0[c];
-                L.v[c] = L.v0[c];
-            }
-        }
-        L.h = A.p.scheme == 1 ? (T)L.tol : (T)A.p.h0;  // fixed step: the line's step (in tol)
-        L.mode = 0;
-        L.tcur = -1;
-        L.tn = 0;
-        acc_reset<T, ACC>(L);
+        start_second<T, ACC, DEV>(A, L);
         return true;
     }
     R.st[L.line] = (uint8_t)L.st;
@@ -1466,7 +1525,9 @@ __device__ __forceinline__ bool init_lattice(const TraceArgs &A, Lane<T> &L, lon
 }
 
 // Rotated extra line q (0: +u, 1: -u, 2: +v, 3: -v) of rotated slot s (Sec. 4).
-template <typename T, bool ACC, bool RECT = false>
+// MERGED: its record follows the lattice's in A.rec (line n + item), else it is
+// line item of A.ext (the same memory).
+template <typename T, bool ACC, bool RECT = false, bool MERGED = false>
 __device__ __forceinline__ bool init_extra(const TraceArgs &A, Lane<T> &L, long long item)
 {
     const Lattice &G = A.lat;
@@ -1494,8 +1555,8 @@ __device__ __forceinline__ bool init_extra(const TraceArgs &A, Lane<T> &L, long 
     double xr[3];
 #pragma unroll
     for (int a = 0; a < 3; a++) xr[a] = state_of<T, RECT>(f, rr[a], a);
-    L.line = item;
-    return start_line<T, ACC, RECT>(A, A.ext, L, xr, nrot, ctl_perp(A.p), 0);
+    L.line = MERGED ? G.n1 * G.n2 * G.n3 + item : item;
+    return start_line<T, ACC, RECT>(A, MERGED ? A.rec : A.ext, L, xr, nrot, ctl_perp(A.p), 0);
 }
 
 template <typename T, bool ACC, bool RECT = false>
@@ -1528,8 +1589,12 @@ __device__ __forceinline__ bool init_list(const TraceArgs &A, Lane<T> &L, long l
 // of the cell it starts in (Sec. 2.3).
 // SCH: 0 = RKF45, 1 = the fixed-step 3/8 rule (every trial accepted; the
 // line's step is held in L.h, halved only by a grazing exit).
+// FLEX: the launch may split directions (DevParams::split) and follow the lattice
+// with extra lines (DevParams::merge); without it neither is looked at, which
+// leaves the hot loop the registers that it had (FP32 map of 1024^2 seeds:
+// 2.05 ms without, 2.25 ms with).
 template <typename T, int SRC, bool ACC, int DEV = 0, bool BATCH = false, bool TAPE = false, bool RECT = false,
-          int SCH = 0>
+          int SCH = 0, bool FLEX = false>
 __device__ __forceinline__ void trace_body(const TraceArgs &A0, const BatchArgs &BA)
 {
     constexpr bool SPLIT = TAPE && SRC == kSrcLattice;
@@ -1541,9 +1606,21 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A0, const BatchArgs 
     const T graze = (T)A0.p.graze;
     const int max_steps = (int)A0.p.max_steps;
 
-    long long nitems = A0.nitems;
-    if (BATCH) nitems = BA.ibase[BA.nent];
-    else if (SRC == kSrcExtra) nitems = 4LL * (long long)(*(volatile unsigned *)A0.q.rot_count);
+    // FP32 lattices: the seed pre-pass has queued the rotated seeds, so their
+    // extra lines follow the lattice's items in the same launch
+    constexpr bool MERGED = FLEX && SRC == kSrcLattice && DEV == 0;
+    long long nlat = A0.nitems;
+    if (BATCH) nlat = BA.ibase[BA.nent];
+    long long nitems = nlat;
+    if (SRC == kSrcExtra && !BATCH) nitems = 4LL * (long long)(*(volatile unsigned *)A0.q.rot_count);
+    if (MERGED && A0.p.merge)
+        nitems += BATCH ? BA.xbase[BA.nent] : 4LL * (long long)(*(volatile unsigned *)A0.q.rot_count);
+    // p.split: 32 items' first directions, then the same 32 items' second ones
+    const bool psplit = FLEX && A0.p.split;
+    if (psplit) nitems = 2 * ((nitems + 31) & ~31LL);
+    // lanes of the warp that take lines (fewer than 32 where the lines would
+    // not fill the GPU's warps; see api.cu)
+    const unsigned gmask = A0.p.lanes >= 32 ? FULL : (1u << A0.p.lanes) - 1u;
 
     long long ck_cur = 0, ck_end = 0, ck_base = 0;
     int ck_ent = 0;
@@ -1562,12 +1639,12 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A0, const BatchArgs 
     for (;;) {
         // refill idle lanes from the warp's chunk / the global counter, once
         // at least p.refill lanes are idle (or none is busy)
-        unsigned idle = __ballot_sync(FULL, !active);
-        const bool refill = __popc(idle) >= A0.p.refill || idle == FULL;
+        unsigned idle = __ballot_sync(FULL, !active) & gmask;
+        const bool refill = __popc(idle) >= A0.p.refill || idle == gmask;
         while (refill && idle != 0u && !exhausted) {
             if (ck_cur >= ck_end) {
                 unsigned long long base = 0;
-                const long long chunk = BATCH ? (long long)kChunk : (long long)A0.p.chunk;
+                const long long chunk = A0.p.chunk;  // (at most 32 with BATCH or p.split)
                 if (lane == 0) base = atomicAdd(A0.q.head, (unsigned long long)chunk);
                 base = __shfl_sync(FULL, base, 0);
                 if ((long long)base >= nitems) {
@@ -1578,24 +1655,28 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A0, const BatchArgs 
                 ck_end = min(ck_cur + chunk, nitems);
                 ck_base = 0;
                 if constexpr (BATCH) {
-                    // entry holding this chunk (chunks never span entries)
+                    // entry holding this chunk (32-item groups never span entries)
+                    long long first = psplit ? ((ck_cur >> 6) << 5) | (ck_cur & 31) : ck_cur;
+                    const bool ext = MERGED && first >= nlat;
+                    const long long *ib = ext ? BA.xbase : BA.ibase;
+                    if (ext) first -= nlat;
                     int lo = 0, hi = BA.nent - 1;
                     while (lo < hi) {
                         const int mid = (lo + hi + 1) >> 1;
-                        if (BA.ibase[mid] <= ck_cur) lo = mid;
+                        if (ib[mid] <= first) lo = mid;
                         else hi = mid - 1;
                     }
                     ck_ent = lo;
-                    ck_base = BA.ibase[lo];
+                    ck_base = ib[lo];
                 }
             }
             const long long avail = ck_end - ck_cur;
             const int rank = __popc(idle & lt_mask);
-            if (!active && rank < avail) {
-                const long long item = ck_cur + rank - ck_base;
+            if (((idle >> lane) & 1u) && rank < avail) {
+                const long long item = ck_cur + rank;
                 eb = ck_ent;
                 const TraceArgs &E = ent();
-                if (SRC == kSrcLattice) {
+                if constexpr (SRC == kSrcLattice) {
                     if constexpr (SPLIT) {
                         // items come in 32-lane groups: a tile's direction 0,
                         // then the same tile's direction 1
@@ -1603,15 +1684,34 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A0, const BatchArgs 
                         active = init_lattice<T, ACC, DEV, RECT>(E, L, ((g >> 1) << 5) | (item & 31), (g & 1) == 0);
                         if (active && (g & 1)) L.end = 1;
                     } else {
-                        active = init_lattice<T, ACC, DEV, RECT>(E, L, item);
+                        const long long slot = psplit ? ((item >> 6) << 5) | (item & 31) : item;
+                        int fl = psplit ? kLaneSplit : 0;
+                        if (!MERGED || slot < nlat) {
+                            active = init_lattice<T, ACC, DEV, RECT>(E, L, slot - ck_base);
+                        } else if constexpr (MERGED) {
+                            const long long x = slot - nlat - ck_base;
+                            fl |= kLaneExtra;
+                            active = x < 4LL * (long long)*E.q.rot_count && init_extra<T, ACC, RECT, true>(E, L, x);
+                        }
+                        if (FLEX && active) {
+                            L.st |= fl;
+                            if (psplit && ((item >> 5) & 1)) L.end = 1;
+                        }
+                    }
+                } else if constexpr (SRC == kSrcExtra) {
+                    const long long x = item - ck_base;
+                    active = x < 4LL * (long long)*E.q.rot_count && init_extra<T, ACC, RECT>(E, L, x);
+                } else {
+                    const long long slot = psplit ? ((item >> 6) << 5) | (item & 31) : item;
+                    active = slot < nlat && init_list<T, ACC, RECT>(E, L, slot);
+                    if (active && psplit) {
+                        L.st |= kLaneSplit;
+                        if ((item >> 5) & 1) L.end = 1;
                     }
                 }
-                else if (SRC == kSrcExtra)
-                    active = item < 4LL * (long long)*E.q.rot_count && init_extra<T, ACC, RECT>(E, L, item);
-                else active = init_list<T, ACC, RECT>(E, L, item);
             }
             ck_cur += min((long long)__popc(idle), avail);
-            idle = __ballot_sync(FULL, !active);
+            idle = __ballot_sync(FULL, !active) & gmask;
         }
         if (__ballot_sync(FULL, active) == 0u) break;
         if (A0.p.sync_dirs) {
@@ -1644,8 +1744,7 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A0, const BatchArgs 
         T hh;
         if (!henon) {
             if (L.steps >= max_steps) {
-                finish_bad<T, SPLIT, RECT>(A, R, L, FQSL_LINE_MAXSTEPS);
-                active = false;
+                active = finish_bad<T, ACC, DEV, SPLIT, RECT, FLEX>(A, R, L, FQSL_LINE_MAXSTEPS);
                 continue;
             }
             hh = L.h;
@@ -1755,8 +1854,7 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A0, const BatchArgs 
         }
 
         if (fail == 1) {
-            finish_bad<T, SPLIT, RECT>(A, R, L, FQSL_LINE_NULL_B);
-            active = false;
+            active = finish_bad<T, ACC, DEV, SPLIT, RECT, FLEX>(A, R, L, FQSL_LINE_NULL_B);
             continue;
         }
         if (!henon) {
@@ -1915,7 +2013,7 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A0, const BatchArgs 
                     ev[c] = L.v[c] + L.t0 * (L.ov[c] - L.v[c]);
                 }
             }
-            active = finish_dir<T, ACC, DEV, SPLIT, RECT>(A, R, L, ex, ey, ez, L.fc0, eu, ev);
+            active = finish_dir<T, ACC, DEV, SPLIT, RECT, FLEX>(A, R, L, ex, ey, ez, L.fc0, eu, ev);
             waiting = active && A0.p.sync_dirs;
             continue;
         }
@@ -1953,7 +2051,7 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A0, const BatchArgs 
                 ev[c] = L.v[c] + hh * ad[3 + c];
             }
         }
-        active = finish_dir<T, ACC, DEV, SPLIT, RECT>(A, R, L, tx, ty, tz, L.hface, eu, ev);
+        active = finish_dir<T, ACC, DEV, SPLIT, RECT, FLEX>(A, R, L, tx, ty, tz, L.hface, eu, ev);
         waiting = active && A0.p.sync_dirs;
     }
 }

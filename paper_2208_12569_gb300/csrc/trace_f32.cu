@@ -14,10 +14,10 @@ namespace fqsl {
 namespace {
 constexpr int kBlock = 128;
 
-template <int SRC, bool ACC>
+template <int SRC, bool ACC, bool FLEX>
 __global__ void __launch_bounds__(kBlock, FQSL_TRACE_F32_MINB) k_trace_f32(const TraceArgs A)
 {
-    trace::trace_body<float, SRC, ACC>(A, BatchArgs{});
+    trace::trace_body<float, SRC, ACC, 0, false, false, false, 0, FLEX>(A, BatchArgs{});
 }
 }  // namespace
 
@@ -25,9 +25,11 @@ namespace {
 template <bool ACC>
 void launch(const TraceArgs &a, int src, int grid, int block, cudaStream_t s)
 {
-    if (src == kSrcLattice) k_trace_f32<kSrcLattice, ACC><<<grid, block, 0, s>>>(a);
-    else if (src == kSrcExtra) k_trace_f32<kSrcExtra, ACC><<<grid, block, 0, s>>>(a);
-    else k_trace_f32<kSrcList, ACC><<<grid, block, 0, s>>>(a);
+    const bool flex = a.p.split || a.p.merge;
+    if (src == kSrcLattice && flex) k_trace_f32<kSrcLattice, ACC, true><<<grid, block, 0, s>>>(a);
+    else if (src == kSrcLattice) k_trace_f32<kSrcLattice, ACC, false><<<grid, block, 0, s>>>(a);
+    else if (flex) k_trace_f32<kSrcList, ACC, true><<<grid, block, 0, s>>>(a);
+    else k_trace_f32<kSrcList, ACC, false><<<grid, block, 0, s>>>(a);
 }
 
 template <bool ACC>
@@ -35,11 +37,9 @@ int blocks(int src)
 {
     int b = 0;
     if (src == kSrcLattice)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_trace_f32<kSrcLattice, ACC>, kBlock, 0);
-    else if (src == kSrcExtra)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_trace_f32<kSrcExtra, ACC>, kBlock, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_trace_f32<kSrcLattice, ACC, true>, kBlock, 0);
     else
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_trace_f32<kSrcList, ACC>, kBlock, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_trace_f32<kSrcList, ACC, true>, kBlock, 0);
     return b > 0 ? b : 1;
 }
 }  // namespace
@@ -86,10 +86,10 @@ cudaError_t launch_seed_prep_f32(const TraceArgs &a, long long n, cudaStream_t s
 
 namespace fqsl {
 namespace {
-template <int WAY>
+template <int WAY, bool FLEX>
 __global__ void __launch_bounds__(kBlock) k_trace_dev_f32(const TraceArgs A)
 {
-    trace::trace_body<float, kSrcLattice, false, WAY>(A, BatchArgs{});
+    trace::trace_body<float, kSrcLattice, false, WAY, false, false, false, 0, FLEX>(A, BatchArgs{});
 }
 }  // namespace
 
@@ -99,16 +99,19 @@ cudaError_t launch_trace_dev_f32(const TraceArgs &a, int way, int grid, int bloc
     if (a.p.scheme == 1)
         return a.f.rect ? launch_trace_dev_rect_rk38_f32(a, way, grid, s) : launch_trace_dev_rk38_f32(a, way, grid, s);
     if (a.f.rect) return launch_trace_dev_rect_f32(a, way, grid, s);
-    if (way == 1) k_trace_dev_f32<1><<<grid, block, 0, s>>>(a);
-    else k_trace_dev_f32<2><<<grid, block, 0, s>>>(a);
+    const bool flex = a.p.split != 0;
+    if (way == 1 && flex) k_trace_dev_f32<1, true><<<grid, block, 0, s>>>(a);
+    else if (way == 1) k_trace_dev_f32<1, false><<<grid, block, 0, s>>>(a);
+    else if (flex) k_trace_dev_f32<2, true><<<grid, block, 0, s>>>(a);
+    else k_trace_dev_f32<2, false><<<grid, block, 0, s>>>(a);
     return cudaGetLastError();
 }
 
 int trace_dev_blocks_per_sm_f32(int way)
 {
     int b = 0;
-    if (way == 1) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_trace_dev_f32<1>, kBlock, 0);
-    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_trace_dev_f32<2>, kBlock, 0);
+    if (way == 1) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_trace_dev_f32<1, false>, kBlock, 0);
+    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_trace_dev_f32<2, false>, kBlock, 0);
     return b > 0 ? b : 1;
 }
 }  // namespace fqsl
@@ -118,10 +121,10 @@ int trace_dev_blocks_per_sm_f32(int way)
 // ---------------------------------------------------------------------------
 namespace fqsl {
 namespace {
-template <int SRC, bool ACC>
+template <bool ACC, bool FLEX>
 __global__ void __launch_bounds__(kBlock, FQSL_TRACE_F32_MINB) k_batch_trace_f32(const TraceArgs A0, const BatchArgs B)
 {
-    trace::trace_body<float, SRC, ACC, 0, true>(A0, B);
+    trace::trace_body<float, kSrcLattice, ACC, 0, true, false, false, 0, FLEX>(A0, B);
 }
 
 __global__ void __launch_bounds__(256) k_batch_seed_prep_f32(const TraceArgs *__restrict__ desc,
@@ -173,17 +176,16 @@ cudaError_t launch_batch_extra_prefix(const unsigned *rot_counts, int nent, long
     return cudaGetLastError();
 }
 
-cudaError_t launch_batch_trace_f32(const TraceArgs &a0, const BatchArgs &b, int src, bool acc64, int grid,
+cudaError_t launch_batch_trace_f32(const TraceArgs &a0, const BatchArgs &b, bool acc64, int grid,
                                    cudaStream_t s)
 {
-    if (a0.p.scheme == 1) return launch_batch_trace_rk38_f32(a0, b, src, acc64, grid, s);
-    if (src == kSrcLattice) {
-        if (acc64) k_batch_trace_f32<kSrcLattice, true><<<grid, kBlock, 0, s>>>(a0, b);
-        else k_batch_trace_f32<kSrcLattice, false><<<grid, kBlock, 0, s>>>(a0, b);
-    } else {
-        if (acc64) k_batch_trace_f32<kSrcExtra, true><<<grid, kBlock, 0, s>>>(a0, b);
-        else k_batch_trace_f32<kSrcExtra, false><<<grid, kBlock, 0, s>>>(a0, b);
-    }
+    if (a0.p.scheme == 1) return launch_batch_trace_rk38_f32(a0, b, acc64, grid, s);
+    // (the extra lines of rotated seeds run in the same launch: DevParams::merge)
+    const bool flex = a0.p.merge != 0;
+    if (acc64 && flex) k_batch_trace_f32<true, true><<<grid, kBlock, 0, s>>>(a0, b);
+    else if (acc64) k_batch_trace_f32<true, false><<<grid, kBlock, 0, s>>>(a0, b);
+    else if (flex) k_batch_trace_f32<false, true><<<grid, kBlock, 0, s>>>(a0, b);
+    else k_batch_trace_f32<false, false><<<grid, kBlock, 0, s>>>(a0, b);
     return cudaGetLastError();
 }
 
@@ -191,8 +193,8 @@ int batch_trace_blocks_per_sm_f32(bool acc64, int scheme)
 {
     if (scheme == 1) return batch_trace_rk38_blocks_per_sm_f32(acc64);
     int b = 0;
-    if (acc64) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_batch_trace_f32<kSrcLattice, true>, kBlock, 0);
-    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_batch_trace_f32<kSrcLattice, false>, kBlock, 0);
+    if (acc64) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_batch_trace_f32<true, true>, kBlock, 0);
+    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_batch_trace_f32<false, true>, kBlock, 0);
     return b > 0 ? b : 1;
 }
 }  // namespace fqsl

@@ -13,25 +13,27 @@ namespace fqsl {
 namespace {
 constexpr int kBlock = 128;
 
-template <int SRC, bool ACC>
+template <int SRC, bool ACC, bool FLEX>
 __global__ void __launch_bounds__(kBlock, FQSL_TRACE_F32_MINB) k_trace_rect_f32(const TraceArgs A)
 {
-    trace::trace_body<float, SRC, ACC, 0, false, false, true>(A, BatchArgs{});
+    trace::trace_body<float, SRC, ACC, 0, false, false, true, 0, FLEX>(A, BatchArgs{});
 }
 
 // Method II (deviation vectors) on a stretched grid
-template <int WAY>
+template <int WAY, bool FLEX>
 __global__ void __launch_bounds__(kBlock) k_trace_dev_rect_f32(const TraceArgs A)
 {
-    trace::trace_body<float, kSrcLattice, false, WAY, false, false, true>(A, BatchArgs{});
+    trace::trace_body<float, kSrcLattice, false, WAY, false, false, true, 0, FLEX>(A, BatchArgs{});
 }
 
 template <bool ACC>
 void launch(const TraceArgs &a, int src, int grid, cudaStream_t s)
 {
-    if (src == kSrcLattice) k_trace_rect_f32<kSrcLattice, ACC><<<grid, kBlock, 0, s>>>(a);
-    else if (src == kSrcExtra) k_trace_rect_f32<kSrcExtra, ACC><<<grid, kBlock, 0, s>>>(a);
-    else k_trace_rect_f32<kSrcList, ACC><<<grid, kBlock, 0, s>>>(a);
+    const bool flex = a.p.split || a.p.merge;
+    if (src == kSrcLattice && flex) k_trace_rect_f32<kSrcLattice, ACC, true><<<grid, kBlock, 0, s>>>(a);
+    else if (src == kSrcLattice) k_trace_rect_f32<kSrcLattice, ACC, false><<<grid, kBlock, 0, s>>>(a);
+    else if (flex) k_trace_rect_f32<kSrcList, ACC, true><<<grid, kBlock, 0, s>>>(a);
+    else k_trace_rect_f32<kSrcList, ACC, false><<<grid, kBlock, 0, s>>>(a);
 }
 
 template <bool ACC>
@@ -39,11 +41,9 @@ int blocks(int src)
 {
     int b = 0;
     if (src == kSrcLattice)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_trace_rect_f32<kSrcLattice, ACC>, kBlock, 0);
-    else if (src == kSrcExtra)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_trace_rect_f32<kSrcExtra, ACC>, kBlock, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_trace_rect_f32<kSrcLattice, ACC, true>, kBlock, 0);
     else
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_trace_rect_f32<kSrcList, ACC>, kBlock, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_trace_rect_f32<kSrcList, ACC, true>, kBlock, 0);
     return b > 0 ? b : 1;
 }
 
@@ -73,16 +73,19 @@ int trace_rect_blocks_per_sm_f32(int src, bool acc64) { return acc64 ? blocks<tr
 
 cudaError_t launch_trace_dev_rect_f32(const TraceArgs &a, int way, int grid, cudaStream_t s)
 {
-    if (way == 1) k_trace_dev_rect_f32<1><<<grid, kBlock, 0, s>>>(a);
-    else k_trace_dev_rect_f32<2><<<grid, kBlock, 0, s>>>(a);
+    const bool flex = a.p.split != 0;
+    if (way == 1 && flex) k_trace_dev_rect_f32<1, true><<<grid, kBlock, 0, s>>>(a);
+    else if (way == 1) k_trace_dev_rect_f32<1, false><<<grid, kBlock, 0, s>>>(a);
+    else if (flex) k_trace_dev_rect_f32<2, true><<<grid, kBlock, 0, s>>>(a);
+    else k_trace_dev_rect_f32<2, false><<<grid, kBlock, 0, s>>>(a);
     return cudaGetLastError();
 }
 
 int trace_dev_rect_blocks_per_sm_f32(int way)
 {
     int b = 0;
-    if (way == 1) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_trace_dev_rect_f32<1>, kBlock, 0);
-    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_trace_dev_rect_f32<2>, kBlock, 0);
+    if (way == 1) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_trace_dev_rect_f32<1, false>, kBlock, 0);
+    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_trace_dev_rect_f32<2, false>, kBlock, 0);
     return b > 0 ? b : 1;
 }
 
