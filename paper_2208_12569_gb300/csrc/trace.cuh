@@ -245,6 +245,22 @@ __device__ __forceinline__ void load_rec32_b(const char *p, float &b0, float &b1
 // runs on GB300's narrow FP64 pipe; this is one FADD and one integer op.)
 __device__ __forceinline__ int small_int(float c) { return __float_as_int(c + 8388608.f) - 0x4B000000; }
 
+template <typename T>
+__device__ __forceinline__ T sel3(int a, T v0, T v1, T v2)
+{
+    return a == 0 ? v0 : (a == 1 ? v1 : v2);
+}
+
+// What an FP32 evaluation read around its point, kept for evaluations a small
+// offset away (Method II way 2): the cell per axis (stretched grid: its record
+// too), the weights and B at the cell's 8 corners in the order of the sum.
+struct Near32 {
+    float c[3];
+    float4 r[3];
+    float w[3], u[3];
+    float b[8][3];
+};
+
 // FP32: weights as products of per-axis weights, corners grouped by (y, z);
 // 32-bit cell arithmetic and byte strides (field_create keeps every axis below
 // 2^23 nodes and the cube below 2^31 nodes; sz32 = 0 marks a z stride that
@@ -252,8 +268,17 @@ __device__ __forceinline__ int small_int(float c) { return __float_as_int(c + 83
 // The 8 corners of cell node (its lowest corner) with per-axis weights w (the
 // upper node's) and u = 1 - w. wj = false: B only (J = 0), half the bytes.
 __device__ __forceinline__ void gather_cell32(const FieldView &f, unsigned node, float wx, float wy, float wz,
-                                              float ux, float uy, float uz, float B[3], float J[3], bool wj = true)
+                                              float ux, float uy, float uz, float B[3], float J[3], bool wj = true,
+                                              Near32 *keep = nullptr)
 {
+    if (keep) {
+        keep->w[0] = wx;
+        keep->w[1] = wy;
+        keep->w[2] = wz;
+        keep->u[0] = ux;
+        keep->u[1] = uy;
+        keep->u[2] = uz;
+    }
     const char *p00 = (const char *)f.rec + (size_t)node * 32u;
     const size_t szb = f.sz32 ? (size_t)f.sz32 : (size_t)f.nx * (size_t)f.ny * 32u;
     const char *pc[4] = {p00, p00 + f.sy32, p00 + szb, p00 + szb + f.sy32};
@@ -270,6 +295,11 @@ __device__ __forceinline__ void gather_cell32(const FieldView &f, unsigned node,
             float r0, r1, r2, r3 = 0.f, r4 = 0.f, r5 = 0.f;
             if (wj) load_rec32(pc[qp] + 32 * m, r0, r1, r2, r3, r4, r5);
             else load_rec32_b(pc[qp] + 32 * m, r0, r1, r2);
+            if (keep) {
+                keep->b[2 * qp + m][0] = r0;
+                keep->b[2 * qp + m][1] = r1;
+                keep->b[2 * qp + m][2] = r2;
+            }
             const float w = (m ? wx : ux) * wyz[qp];
             B[0] += w * r0;
             B[1] += w * r1;
@@ -283,8 +313,40 @@ __device__ __forceinline__ void gather_cell32(const FieldView &f, unsigned node,
     }
 }
 
+// B at the kept point moved to xa along axis a, from the kept corners if that is
+// still in the kept cell (the same sum as gather_cell32's, so the same B), else
+// by a gather of its own. RECT: a stretched grid.
+template <bool RECT>
+__device__ __forceinline__ bool gather_near(const FieldView &f, const Near32 &n, int a, float xa, float B[3])
+{
+    float w, u;
+    if constexpr (RECT) {
+        const float r0 = sel3(a, n.r[0].x, n.r[1].x, n.r[2].x), r1 = sel3(a, n.r[0].y, n.r[1].y, n.r[2].y);
+        if (!(xa >= r0 && xa < r1)) return false;
+        u = (r1 - xa) * sel3(a, n.r[0].z, n.r[1].z, n.r[2].z);
+        w = 1.f - u;
+    } else {
+        const float c = fminf(fmaxf(floorf(xa), 0.f), sel3(a, f.cmax[0], f.cmax[1], f.cmax[2]));
+        if (c != sel3(a, n.c[0], n.c[1], n.c[2])) return false;
+        w = xa - c;
+        u = 1.f - w;
+    }
+    const float wx = a == 0 ? w : n.w[0], wy = a == 1 ? w : n.w[1], wz = a == 2 ? w : n.w[2];
+    const float ux = a == 0 ? u : n.u[0], uy = a == 1 ? u : n.u[1], uz = a == 2 ? u : n.u[2];
+    const float wyz[4] = {uy * uz, wy * uz, uy * wz, wy * wz};
+#pragma unroll
+    for (int c = 0; c < 3; c++) B[c] = 0.f;
+#pragma unroll
+    for (int q = 0; q < 8; q++) {
+        const float wt = ((q & 1) ? wx : ux) * wyz[q >> 1];
+#pragma unroll
+        for (int c = 0; c < 3; c++) B[c] += wt * n.b[q][c];
+    }
+    return true;
+}
+
 __device__ __forceinline__ void gather(const FieldView &f, float x, float y, float z, float B[3], float J[3],
-                                       bool wj = true)
+                                       bool wj = true, Near32 *keep = nullptr)
 {
     const float cx = fminf(fmaxf(floorf(x), 0.f), f.cmax[0]);
     const float cy = fminf(fmaxf(floorf(y), 0.f), f.cmax[1]);
@@ -293,7 +355,12 @@ __device__ __forceinline__ void gather(const FieldView &f, float x, float y, flo
     const float ux = 1.f - wx, uy = 1.f - wy, uz = 1.f - wz;
     const unsigned node = ((unsigned)small_int(cz) * (unsigned)f.ny + (unsigned)small_int(cy)) * (unsigned)f.nx +
                           (unsigned)small_int(cx);
-    gather_cell32(f, node, wx, wy, wz, ux, uy, uz, B, J, wj);
+    if (keep) {
+        keep->c[0] = cx;
+        keep->c[1] = cy;
+        keep->c[2] = cz;
+    }
+    gather_cell32(f, node, wx, wy, wz, ux, uy, uz, B, J, wj, keep);
 }
 
 // FP64: Eq. interp term by term, omega_0 = (i+1) - xi and omega_1 = 1 - omega_0
@@ -424,12 +491,16 @@ __device__ __forceinline__ void rect_cells(const FieldView &f, T x, T y, T z, Re
 // FP32 on a stretched grid: state coordinates relative to the first node,
 // omega_0 = (x_{i+1} - x) / (x_{i+1} - x_i) with the reciprocal width (Eq. w0)
 __device__ __forceinline__ void gather_rect_at(const FieldView &f, float x, float y, float z, const RectCells<float> &rc,
-                                               float B[3], float J[3], bool wj = true)
+                                               float B[3], float J[3], bool wj = true, Near32 *keep = nullptr)
 {
+    if (keep) {
+#pragma unroll
+        for (int a = 0; a < 3; a++) keep->r[a] = rc.r[a];
+    }
     const float ux = (rc.r[0].y - x) * rc.r[0].z, uy = (rc.r[1].y - y) * rc.r[1].z, uz = (rc.r[2].y - z) * rc.r[2].z;
     const unsigned node =
         ((unsigned)rc.c[2] * (unsigned)f.ny + (unsigned)rc.c[1]) * (unsigned)f.nx + (unsigned)rc.c[0];
-    gather_cell32(f, node, 1.f - ux, 1.f - uy, 1.f - uz, ux, uy, uz, B, J, wj);
+    gather_cell32(f, node, 1.f - ux, 1.f - uy, 1.f - uz, ux, uy, uz, B, J, wj, keep);
 }
 
 // FP64 on a stretched grid: Eqs. interp, w0, w1 as written in physical
@@ -550,10 +621,10 @@ __device__ __forceinline__ double state_of(const FieldView &f, double r, int a)
 // Returns false on a null / non-finite field. wj = false (a stage whose Tw
 // weight is zero): dTw/dtau = 0 without loading curl B.
 __device__ __forceinline__ bool rhs(const FieldView &f, const float invd[3], float sgn, float x, float y, float z,
-                                    float out[5], bool wj = true)
+                                    float out[5], bool wj = true, Near32 *keep = nullptr)
 {
     float B[3], J[3];
-    gather(f, x, y, z, B, J, wj);
+    gather(f, x, y, z, B, J, wj, keep);
     const float b0 = B[0] * invd[0], b1 = B[1] * invd[1], b2 = B[2] * invd[2];
     const float bb = b0 * b0 + b1 * b1 + b2 * b2;
     const float BB = B[0] * B[0] + B[1] * B[1] + B[2] * B[2];
@@ -574,7 +645,7 @@ __device__ __forceinline__ bool rhs(const FieldView &f, const float invd[3], flo
 // dTw/dtau = (J.B) / (4 pi B^2) dl/dtau, each as written.
 // (wj: accepted for the common interface; FP64 always forms dTw/dtau)
 __device__ __forceinline__ bool rhs(const FieldView &f, const double d[3], double sgn, double x, double y,
-                                    double z, double out[5], bool wj = true)
+                                    double z, double out[5], bool wj = true, Near32 * = nullptr)
 {
     double B[3], J[3];
     gather(f, x, y, z, B, J);
@@ -596,11 +667,17 @@ __device__ __forceinline__ bool rhs(const FieldView &f, const double d[3], doubl
 // Stretched grid: bt_a = B_a / D_a with the step's cell widths D, and the
 // physical velocity F = sigma B / |bt| (FP32: rw = 1/D).
 __device__ __forceinline__ bool rhs_rect(const FieldView &f, const float rw[3], float sgn, float x, float y, float z,
-                                         float out[5], const RectCells<float> *pre = nullptr, bool wj = true)
+                                         float out[5], const RectCells<float> *pre = nullptr, bool wj = true,
+                                         Near32 *keep = nullptr)
 {
     float B[3], J[3];
-    if (pre) gather_rect_at(f, x, y, z, *pre, B, J, wj);
-    else gather_rect(f, x, y, z, B, J, wj);
+    if (pre) {
+        gather_rect_at(f, x, y, z, *pre, B, J, wj, keep);
+    } else {
+        RectCells<float> rc;
+        rect_cells(f, x, y, z, rc);
+        gather_rect_at(f, x, y, z, rc, B, J, wj, keep);
+    }
     const float b0 = B[0] * rw[0], b1 = B[1] * rw[1], b2 = B[2] * rw[2];
     const float bb = b0 * b0 + b1 * b1 + b2 * b2;
     const float BB = B[0] * B[0] + B[1] * B[1] + B[2] * B[2];
@@ -619,7 +696,7 @@ __device__ __forceinline__ bool rhs_rect(const FieldView &f, const float rw[3], 
 
 __device__ __forceinline__ bool rhs_rect(const FieldView &f, const double D[3], double sgn, double x, double y,
                                          double z, double out[5], const RectCells<double> *pre = nullptr,
-                                         bool wj = true)
+                                         bool wj = true, Near32 * = nullptr)
 {
     double B[3], J[3];
     if (pre) gather_rect_at(f, x, y, z, *pre, B, J);
@@ -641,10 +718,10 @@ __device__ __forceinline__ bool rhs_rect(const FieldView &f, const double D[3], 
 // pre (stretched grid): the point's cells, already searched
 template <bool RECT, typename T>
 __device__ __forceinline__ bool rhsg(const FieldView &f, const T dd[3], T sgn, T x, T y, T z, T out[5],
-                                     const RectCells<T> *pre = nullptr, bool wj = true)
+                                     const RectCells<T> *pre = nullptr, bool wj = true, Near32 *keep = nullptr)
 {
-    if constexpr (RECT) return rhs_rect(f, dd, sgn, x, y, z, out, pre, wj);
-    else return rhs(f, dd, sgn, x, y, z, out, wj);
+    if constexpr (RECT) return rhs_rect(f, dd, sgn, x, y, z, out, pre, wj, keep);
+    else return rhs(f, dd, sgn, x, y, z, out, wj, keep);
 }
 
 // ---------------------------------------------------------------------------
@@ -800,13 +877,6 @@ __device__ __forceinline__ bool grad_bhat(const FieldView &f, T eps, T x, T y, T
             }
             xp[a] += off;
             xm[a] -= off;
-            if constexpr (sizeof(T) == 4) {
-                // FP32: divide by the offset the rounded positions realise (their
-                // difference is exact); at x ~ 255 cells a float moves in steps
-                // of 1.5e-5 cells, 1.5 % of a 0.001-cell offset
-                const T h = xp[a] - xm[a];
-                span = RECT ? h : h * (T)f.d[a];
-            }
             T bp[3], bm[3];
             ok &= unit_b<T, RECT>(f, xp[0], xp[1], xp[2], bp);
             ok &= unit_b<T, RECT>(f, xm[0], xm[1], xm[2], bm);
@@ -815,6 +885,72 @@ __device__ __forceinline__ bool grad_bhat(const FieldView &f, T eps, T x, T y, T
         }
         return ok;
     }
+}
+
+// (U . grad)(B/|B|) and (V . grad)(B/|B|) by way 2 in FP32: us = {U, V}, near = what
+// the evaluation at (x, y, z) read. The offset points lie in its cell nearly
+// always (eps is 0.001 cells), so B there is formed from the corners in
+// registers instead of gathered again: a stage loads 8 records, not 56. Points
+// that left the cell gather for themselves, in one loop behind the six (a
+// gather inlined behind each outgrew the instruction cache: 5.0 ms for a map of
+// 384x256 seeds, against 3.57 ms for seven gathers a stage and 2.76 ms in this
+// form; a rolled loop over the axes 2.99 ms, and 1.15 against 0.93 ms for a map
+// of 11,254 seeds, whose warps wait on the loop's chain of divisions).
+// Each difference is divided by the offset that the rounded positions realise
+// (their difference is exact): at x ~ 255 cells a float moves in steps of
+// 1.5e-5 cells, 1.5 % of a 0.001-cell offset.
+template <bool RECT>
+__device__ __forceinline__ bool grad_way2_32(const FieldView &f, float eps, float x, float y, float z,
+                                             const float dd[3], const Near32 &near, const float us[6], float su[3],
+                                             float sv[3])
+{
+    bool ok = true;
+#pragma unroll
+    for (int b = 0; b < 3; b++) su[b] = sv[b] = 0.f;
+    const float p[3] = {x, y, z};
+    float xo[6], B[6][3];
+    unsigned out = 0u;  // points that left the cell
+#pragma unroll
+    for (int t = 0; t < 6; t++) {
+        const float e = (t & 1) ? -eps : eps;
+        xo[t] = p[t >> 1] + e;
+        if constexpr (RECT) xo[t] = fmaf(e, 1.f / dd[t >> 1], p[t >> 1]);
+        if (!gather_near<RECT>(f, near, t >> 1, xo[t], B[t])) out |= 1u << t;
+    }
+#pragma unroll 1
+    while (out) {
+        const int q = __ffs(out) - 1;
+        out &= out - 1u;
+        float xa = xo[0];
+#pragma unroll
+        for (int t = 1; t < 6; t++) xa = q == t ? xo[t] : xa;
+        float C[3], J[3];
+        gatherg<RECT>(f, q < 2 ? xa : x, (q >> 1) == 1 ? xa : y, q > 3 ? xa : z, C, J, false);
+#pragma unroll
+        for (int t = 0; t < 6; t++)
+#pragma unroll
+            for (int c = 0; c < 3; c++) B[t][c] = q == t ? C[c] : B[t][c];
+    }
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        const float h = xo[2 * a] - xo[2 * a + 1];
+        const float span = RECT ? h : h * (float)f.d[a];
+        float m[2];
+#pragma unroll
+        for (int t = 0; t < 2; t++) {
+            const float *b = B[2 * a + t];
+            m[t] = sqrt(b[0] * b[0] + b[1] * b[1] + b[2] * b[2]);
+            const bool fine = m[t] > 0.f && m[t] < INFINITY;
+            ok = ok && fine;
+        }
+#pragma unroll
+        for (int b = 0; b < 3; b++) {
+            const float g = (B[2 * a][b] / m[0] - B[2 * a + 1][b] / m[1]) / span;
+            su[b] += us[a] * g;
+            sv[b] += us[3 + a] * g;
+        }
+    }
+    return ok;
 }
 
 // fourth root through the correctly rounded square root
@@ -864,12 +1000,6 @@ __device__ __forceinline__ bool in_box(const FieldView &f, const double xi[3])
 #pragma unroll
     for (int a = 0; a < 3; a++) in = in && xi[a] >= dlo<T, RECT>(f, a) && xi[a] <= dhi<T, RECT>(f, a);
     return in;
-}
-
-template <typename T>
-__device__ __forceinline__ T sel3(int a, T v0, T v1, T v2)
-{
-    return a == 0 ? v0 : (a == 1 ? v1 : v2);
 }
 
 // Seed position of lattice index (i, j, k) in physical coordinates, evaluated
@@ -1778,7 +1908,9 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A0, const BatchArgs 
             // FP32: RKF45's stages 1 and 5 have zero 4th-order weight, so their
             // Tw integrand is not formed (nor their curl B loaded)
             const bool wj = kF64 || SCH != 0 || (s != 1 && s != 5);
-            bool ok = rhsg<RECT>(f, dd, sgn, px, py, pz, o, (RECT && s == 0) ? &rc0 : nullptr, wj);
+            Near32 near;  // FP32 Method II way 2: what this evaluation read
+            bool ok = rhsg<RECT>(f, dd, sgn, px, py, pz, o, (RECT && s == 0) ? &rc0 : nullptr, wj,
+                                 (DEV == 2 && !kF64) ? &near : nullptr);
             if constexpr (DEV != 0) {
                 // stage deviation vectors and Eq. rb2: dU/dtau = sigma (ds/dtau) (U . grad)(B/|B|)
                 T us[6];
@@ -1789,19 +1921,29 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A0, const BatchArgs 
                     for (int r = 0; r < s; r++) acc += Tab<T, SCH>::a(s, r) * kd[r][c];
                     us[c] = (c < 3 ? L.u[c] : L.v[c - 3]) + hh * acc;
                 }
-                T G[3][3];
-                ok = grad_bhat<T, DEV, RECT>(f, (T)A0.p.eps2, px, py, pz, dd, G) && ok;
                 const T sdl = sgn * o[3];
+                if constexpr (DEV == 2 && !kF64) {
+                    float su[3], sv[3];
+                    ok = grad_way2_32<RECT>(f, (float)A0.p.eps2, px, py, pz, dd, near, us, su, sv) && ok;
 #pragma unroll
-                for (int b = 0; b < 3; b++) {
-                    T su = 0, sv = 0;
-#pragma unroll
-                    for (int a = 0; a < 3; a++) {
-                        su += us[a] * G[a][b];
-                        sv += us[3 + a] * G[a][b];
+                    for (int b = 0; b < 3; b++) {
+                        o[5 + b] = sdl * su[b];
+                        o[8 + b] = sdl * sv[b];
                     }
-                    o[5 + b] = sdl * su;
-                    o[8 + b] = sdl * sv;
+                } else {
+                    T G[3][3];
+                    ok = grad_bhat<T, DEV, RECT>(f, (T)A0.p.eps2, px, py, pz, dd, G) && ok;
+#pragma unroll
+                    for (int b = 0; b < 3; b++) {
+                        T su = 0, sv = 0;
+#pragma unroll
+                        for (int a = 0; a < 3; a++) {
+                            su += us[a] * G[a][b];
+                            sv += us[3 + a] * G[a][b];
+                        }
+                        o[5 + b] = sdl * su;
+                        o[8 + b] = sdl * sv;
+                    }
                 }
             }
             if (!ok && !fail) fail = 1;

@@ -5,6 +5,12 @@
 // per-line tolerance, footpoints and Bn are double in both.
 #include "trace.cuh"
 
+// resident blocks per SM asked of the Method II tracers: 3 (168 registers, a few
+// spills); 2 measured slower (384x256 seeds, way 2: 2.90 against 2.77 ms)
+#ifndef FQSL_TRACE_DEV_F32_MINB
+#define FQSL_TRACE_DEV_F32_MINB 3
+#endif
+
 // minimum resident blocks per SM requested from the register allocator
 #ifndef FQSL_TRACE_F32_MINB
 #define FQSL_TRACE_F32_MINB 4
@@ -87,7 +93,7 @@ cudaError_t launch_seed_prep_f32(const TraceArgs &a, long long n, cudaStream_t s
 namespace fqsl {
 namespace {
 template <int WAY, bool FLEX>
-__global__ void __launch_bounds__(kBlock) k_trace_dev_f32(const TraceArgs A)
+__global__ void __launch_bounds__(kBlock, FQSL_TRACE_DEV_F32_MINB) k_trace_dev_f32(const TraceArgs A)
 {
     trace::trace_body<float, kSrcLattice, false, WAY, false, false, false, 0, FLEX>(A, BatchArgs{});
 }

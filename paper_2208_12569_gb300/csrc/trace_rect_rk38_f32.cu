@@ -3,6 +3,12 @@
 // RECT and the SCH forms. Method I sources and Method II's two ways.
 #include "trace.cuh"
 
+// resident blocks per SM asked of the Method II tracers: 3 (168 registers, a few
+// spills); 2 measured slower (384x256 seeds, way 2: 2.90 against 2.77 ms)
+#ifndef FQSL_TRACE_DEV_F32_MINB
+#define FQSL_TRACE_DEV_F32_MINB 3
+#endif
+
 #ifndef FQSL_TRACE_F32_MINB
 #define FQSL_TRACE_F32_MINB 4
 #endif
@@ -18,7 +24,7 @@ __global__ void __launch_bounds__(kBlock, FQSL_TRACE_F32_MINB) k_trace_rect_rk38
 }
 
 template <int WAY, bool FLEX>
-__global__ void __launch_bounds__(kBlock) k_trace_dev_rect_rk38_f32(const TraceArgs A)
+__global__ void __launch_bounds__(kBlock, FQSL_TRACE_DEV_F32_MINB) k_trace_dev_rect_rk38_f32(const TraceArgs A)
 {
     trace::trace_body<float, kSrcLattice, false, WAY, false, false, true, 1, FLEX>(A, BatchArgs{});
 }
