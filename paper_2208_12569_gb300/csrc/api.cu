@@ -644,9 +644,12 @@ int tlb_blocks(size_t record_bytes, SeedKind kind, bool sparse, int bps)
 //     500 seeds 0.36 -> 0.26 ms with 2 lanes, plane of 4,096 seeds 0.38 -> 0.32
 //     ms with 4, of 40,000 0.58 -> 0.51 ms with 16; with more warps than fit at
 //     once it loses: 90,000 seeds of a plane 0.62 -> 0.84 ms, a list of 40,604
-//     seeds 0.45 -> 0.56 ms). FP64 warp instructions
-//     take the narrow FP64 pipe the same time whatever their lanes, so FP64
-//     lines are spread only over SMs that would idle.
+//     seeds 0.45 -> 0.56 ms). The FP64 tracer of Method I gives a line eight
+//     lanes, so four lines fill a warp. FP64 Method II lines, one per lane, are
+//     spread only over SMs that would idle: their warp instructions take the
+//     narrow FP64 pipe the same time whatever their lanes.
+int lanes_per_line(const fqsl_params *p) { return p->precision == FQSL_F64 && p->method == 1 ? 8 : 1; }
+
 Spread spread_of(const fqsl_field f, const fqsl_params *p, int bps, long long lines, SeedKind kind, bool sparse,
                  bool may_split)
 {
@@ -658,9 +661,10 @@ Spread spread_of(const fqsl_field f, const fqsl_params *p, int bps, long long li
     if (f32 && may_split && kind == kSeedsInside) r.split = lines <= (p->method == 2 ? 16 : 96) * warps;
     if (f32 && may_split && kind == kSeedsList) r.split = 2 * lines <= warps;
     const long long items = (r.split ? 2 : 1) * lines;
-    const long long most = !f32 ? f->sms : (kind == kSeedsFace ? warps + warps / 16 : warps);
-    if (p->chunk_tiles == 0)
-        while (r.lanes > 1 && items <= most * (r.lanes / 2)) r.lanes /= 2;
+    const int per = lanes_per_line(p);
+    const long long most = !f32 && per == 1 ? f->sms : (f32 && kind == kSeedsFace ? warps + warps / 16 : warps);
+    if (p->chunk_tiles == 0 || per > 1)
+        while (r.lanes > per && items <= most * (r.lanes / per / 2)) r.lanes /= 2;
     return r;
 }
 
@@ -795,20 +799,21 @@ int blocks_per_sm(fqsl_field f, int precision, int src, int p_scheme)
 
 // The grid of a launch of `items` items spread as sp says; full: lines that the
 // host cannot count follow (extra lines), so the grid fills the GPU.
-long long spread_grid(const Spread &sp, int sms, long long items, bool full)
+long long spread_grid(const fqsl_params *p, const Spread &sp, int sms, long long items, bool full)
 {
     long long grid = (long long)sms * sp.bps;
-    const long long per_block = (long long)sp.lanes * (kTraceBlock / 32);
+    const long long per_block = (long long)(sp.lanes / lanes_per_line(p)) * (kTraceBlock / 32);
     const long long need = ((sp.split ? 2 : 1) * items + per_block - 1) / per_block;
     if (!full && need < grid) grid = need;
     return grid < 1 ? 1 : grid;
 }
 
-void set_spread(TraceArgs &a, const Spread &sp)
+void set_spread(TraceArgs &a, const fqsl_params *p, const Spread &sp)
 {
     a.p.lanes = sp.lanes;
     a.p.split = sp.split ? 1 : 0;
-    if (sp.lanes < 32) a.p.chunk = sp.lanes;
+    if (lanes_per_line(p) > 1) a.p.chunk = sp.lanes / lanes_per_line(p);
+    else if (sp.lanes < 32) a.p.chunk = sp.lanes;
     else if (sp.split) a.p.chunk = kTileU * kTileV;
 }
 
@@ -830,7 +835,7 @@ cudaError_t launch_extra(fqsl_field f, const fqsl_params *p, TraceArgs a, const 
         a.nitems = 0;
         a.p.merge = 1;
     }
-    return launch_trace(p, a, f32 ? kSrcLattice : kSrcExtra, spread_grid(sp, f->sms, 0, true), stream);
+    return launch_trace(p, a, f32 ? kSrcLattice : kSrcExtra, spread_grid(p, sp, f->sms, 0, true), stream);
 }
 
 int blocks_per_sm_m2(fqsl_field f, const fqsl_params *p)
@@ -1095,7 +1100,7 @@ fqsl_status run_qmap_locked(fqsl_field f, const Lattice &lat0, const fqsl_params
     a.prep = s.prep;
     a.tape = tl.tape;
     a.nitems = lat.n3 * lat.tiles_u * lat.tiles_v * (long long)(kTileU * kTileV);
-    if (!tape) set_spread(a, sp);
+    if (!tape) set_spread(a, p, sp);
     // (with timing on, the extra lines get a launch of their own to be timed)
     a.p.merge = !tape && f32 && rot && !f->timing;
     if (f32) {
@@ -1104,7 +1109,7 @@ fqsl_status run_qmap_locked(fqsl_field f, const Lattice &lat0, const fqsl_params
     }
     mark(f, 0, stream);
     if (m2) {
-        e = launch_trace_m2(p, a, spread_grid(sp, f->sms, a.nitems, false), stream);
+        e = launch_trace_m2(p, a, spread_grid(p, sp, f->sms, a.nitems, false), stream);
         if (e != cudaSuccess) return cuda_fail(e, who);
         mark(f, 1, stream);
         mark(f, 2, stream);
@@ -1128,12 +1133,14 @@ fqsl_status run_qmap_locked(fqsl_field f, const Lattice &lat0, const fqsl_params
         if (p->blocks_per_sm > 0 && p->blocks_per_sm < bps) bps = p->blocks_per_sm;
         long long grid = (long long)f->sms * bps;
         a.nitems *= 2;  // one item per direction of a line
-        const long long need = (a.nitems + kTraceBlock - 1) / kTraceBlock;
+        const int per = lanes_per_line(p);
+        if (per > 1) a.p.chunk = 32 / per;
+        const long long need = (a.nitems * per + kTraceBlock - 1) / kTraceBlock;
         if (need < grid) grid = need;
         if (grid < 1) grid = 1;
         e = launch_tape(a, p, kSrcLattice, grid, stream);
     } else {
-        e = launch_trace(p, a, kSrcLattice, spread_grid(sp, f->sms, a.nitems, a.p.merge != 0), stream);
+        e = launch_trace(p, a, kSrcLattice, spread_grid(p, sp, f->sms, a.nitems, a.p.merge != 0), stream);
     }
     if (e != cudaSuccess) return cuda_fail(e, who);
     mark(f, 1, stream);
@@ -1349,9 +1356,9 @@ fqsl_status fqsl_twist(fqsl_field f, const double *seeds_dev, long long n, const
     a.nitems = n;
     a.rec = s.rec;
     a.q.head = s.ctr;
-    set_spread(a, sp);
+    set_spread(a, p, sp);
     mark(f, 0, stream);
-    e = launch_trace(p, a, kSrcList, spread_grid(sp, f->sms, (n + 31) / 32 * 32, false), stream);
+    e = launch_trace(p, a, kSrcList, spread_grid(p, sp, f->sms, (n + 31) / 32 * 32, false), stream);
     if (e != cudaSuccess) return cuda_fail(e, who);
     mark(f, 1, stream);
     mark(f, 2, stream);
@@ -1500,14 +1507,14 @@ extern "C" fqsl_status fqsl_qmap_plane_static(fqsl_field f, const double origin[
     a.q.rot_slot = s.rot_slot;
     a.prep = s.prep;
     a.nitems = lat.n3 * lat.tiles_u * lat.tiles_v * (long long)(kTileU * kTileV);
-    set_spread(a, sp);
+    set_spread(a, p, sp);
     a.p.merge = f32 && rot && !f->timing;
     if (f32) {
         e = launch_seed_prep_f32(a, n, stream);
         if (e != cudaSuccess) return cuda_fail(e, who);
     }
     mark(f, 0, stream);
-    e = launch_trace(p, a, kSrcLattice, spread_grid(sp, f->sms, a.nitems, a.p.merge != 0), stream);
+    e = launch_trace(p, a, kSrcLattice, spread_grid(p, sp, f->sms, a.nitems, a.p.merge != 0), stream);
     if (e != cudaSuccess) return cuda_fail(e, who);
     mark(f, 1, stream);
     if (rot && !a.p.merge) {
@@ -1749,7 +1756,8 @@ extern "C" fqsl_status fqsl_batch_run(fqsl_batch b, void *cuda_stream)
     if (e != cudaSuccess) return cuda_fail(e, who);
     TraceArgs a0{};
     a0.p = dev_params(p);
-    a0.p.chunk = kTileU * kTileV;  // a grab never spans two entries
+    const int per = lanes_per_line(p);
+    a0.p.chunk = 32 / per;  // a grab never spans two entries
     a0.q.head = b->d_heads;
     a0.nitems = b->total_items;
     a0.p.merge = f32 && b->any_rot;
@@ -1759,7 +1767,7 @@ extern "C" fqsl_status fqsl_batch_run(fqsl_batch b, void *cuda_stream)
     }
     BatchArgs ba{b->d_desc, b->d_ibase, b->nent, b->d_xbase};
     long long grid = b->grid;
-    const long long need = (b->total_items + kTraceBlock - 1) / kTraceBlock;
+    const long long need = (b->total_items * per + kTraceBlock - 1) / kTraceBlock;
     if (!a0.p.merge && need < grid) grid = need;
     e = f32 ? launch_batch_trace_f32(a0, ba, p->precision == FQSL_F32_ACC64, (int)grid, s)
             : launch_batch_trace_f64(a0, ba, kSrcLattice, (int)grid, s);

@@ -1,4 +1,6 @@
-// Persistent field-line tracer (templated on the traced precision T).
+// Persistent field-line tracer (templated on the traced precision T; the FP64
+// maps of Method I and seed lists are traced by trace64.cuh, in the arithmetic
+// that this file states).
 //
 // Method (Zhang et al. 2022):
 //   - field-line equation dr/ds = B/|B| (Sec. 2.1, Eq. rb), integrated in index
@@ -39,15 +41,12 @@
 
 #include "fqsl_internal.cuh"
 
-// Resident 128-thread blocks per SM asked of the FP64 RKF45 tracers (not the
-// Method II or fixed-step ones): their latency (FP64 divisions and square
-// roots on GB300's narrow FP64 pipe) wants warps more than registers. 8 blocks
-// (64 registers, the rest spilled to L1) measured fastest: 92.5 ms per
-// 1024x1024 map of the 256x256x128 monopole cube against 108.9 ms at 168
-// registers and 3 blocks. The fixed-step FP64 map measured slower with it
-// (8.5 against 8.9 M Q+Tw/s) and keeps its registers.
+// Resident 128-thread blocks per SM asked of the FP64 tracers of Method I
+// (trace64.cuh; about 100 registers a lane): 4. At 3, 5, 6 and 8 blocks a map of
+// 512x512 seeds of the 256x256x128 cube took 23.5, 23.6, 25.3 and 25.4 ms
+// against 23.4 ms, smaller maps up to 1.2 times as long at 6 and 8.
 #ifndef FQSL_TRACE_F64_MINB
-#define FQSL_TRACE_F64_MINB 8
+#define FQSL_TRACE_F64_MINB 4
 #endif
 
 namespace fqsl {
@@ -1154,22 +1153,12 @@ __device__ __forceinline__ void store_state(float *p, float x, float y, float z)
 {
     *(float4 *)p = make_float4(x, y, z, 0.f);
 }
-__device__ __forceinline__ void store_state(double *p, double x, double y, double z)
-{
-    ((double2 *)p)[0] = make_double2(x, y);
-    ((double2 *)p)[1] = make_double2(z, 0.0);
-}
 // the first N (a multiple of 4) values of v
 template <typename T, int N>
 __device__ __forceinline__ void store_vec(T *p, const T v[])
 {
-    if constexpr (sizeof(T) == 4) {
 #pragma unroll
-        for (int q = 0; q < N; q += 4) *(float4 *)(p + q) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
-    } else {
-#pragma unroll
-        for (int q = 0; q < N; q += 2) *(double2 *)(p + q) = make_double2(v[q], v[q + 1]);
-    }
+    for (int q = 0; q < N; q += 4) *(float4 *)(p + q) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
 }
 
 // Open a new chunk whose checkpoint is the current state. Returns false when
@@ -1251,21 +1240,12 @@ __device__ __forceinline__ void or_status(uint8_t *st, long long line, unsigned 
 }
 
 template <typename T>
-__device__ __forceinline__ void split_finish(const TraceArgs &A, const LineRecs &R, Lane<T> &L, bool bad)
+__device__ __forceinline__ void split_finish(const TraceArgs &A, const LineRecs &R, Lane<T> &L)
 {
     const int before = atomicAdd(R.steps + L.line, L.steps);
     unsigned st = (unsigned)L.st;
-    if ((long long)before + L.steps > A.p.max_steps) {
-        st |= FQSL_LINE_MAXSTEPS;
-        bad = true;
-    }
+    if ((long long)before + L.steps > A.p.max_steps) st |= FQSL_LINE_MAXSTEPS;
     or_status(R.st, L.line, st);
-    if constexpr (sizeof(T) == 8) {
-        if (bad) {
-            if (R.tw) R.tw[L.line] = NAN;
-            if (R.len) R.len[L.line] = NAN;
-        }
-    }
 }
 
 // Start the second direction of a line at its seed.
@@ -1353,7 +1333,7 @@ __device__ __forceinline__ bool finish_bad(const TraceArgs &A, const LineRecs &R
         }
     }
     if constexpr (SPLIT) {
-        split_finish(A, R, L, true);
+        split_finish(A, R, L);
     } else {
         R.st[L.line] = (uint8_t)L.st;
         R.steps[L.line] = L.steps;
@@ -1412,11 +1392,7 @@ __device__ __forceinline__ bool finish_dir(const TraceArgs &A, const LineRecs &R
         }
     }
     if constexpr (SPLIT) {
-        if constexpr (sizeof(T) == 8) {
-            if (R.tw) atomicAdd(R.tw + L.line, acc_tw<T, ACC>(L));
-            if (R.len) atomicAdd(R.len + L.line, acc_len<T, ACC>(L));
-        }
-        split_finish(A, R, L, false);
+        split_finish(A, R, L);
         return false;
     }
     if constexpr (FLEX) {

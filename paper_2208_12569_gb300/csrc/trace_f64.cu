@@ -1,6 +1,6 @@
 // FP64 instantiation of the persistent tracer: the cube, the line state and all
 // arithmetic are in double (the parity reference of the float tracer).
-#include "trace.cuh"
+#include "trace64.cuh"
 
 namespace fqsl {
 namespace {
@@ -9,7 +9,7 @@ constexpr int kBlock = 128;
 template <int SRC>
 __global__ void __launch_bounds__(kBlock, FQSL_TRACE_F64_MINB) k_trace_f64(const TraceArgs A)
 {
-    trace::trace_body<double, SRC, true>(A, BatchArgs{});
+    trace64::trace_body<SRC, false, false, false, 0>(A, BatchArgs{});
 }
 }  // namespace
 
@@ -70,7 +70,7 @@ namespace {
 template <int SRC>
 __global__ void __launch_bounds__(kBlock, FQSL_TRACE_F64_MINB) k_batch_trace_f64(const TraceArgs A0, const BatchArgs B)
 {
-    trace::trace_body<double, SRC, true, 0, true>(A0, B);
+    trace64::trace_body<SRC, true, false, false, 0>(A0, B);
 }
 }  // namespace
 
@@ -97,7 +97,7 @@ namespace {
 template <int SRC>
 __global__ void __launch_bounds__(kBlock, FQSL_TRACE_F64_MINB) k_trace_tape_f64(const TraceArgs A)
 {
-    trace::trace_body<double, SRC, true, 0, false, true>(A, BatchArgs{});
+    trace64::trace_body<SRC, false, true, false, 0>(A, BatchArgs{});
 }
 }  // namespace
 

@@ -3,7 +3,7 @@
 // written and per-cell step and error scaling (trace_body's RECT form). Built
 // without contraction like trace_f64.cu, so that it reproduces a plain
 // evaluation of the method to the last bit.
-#include "trace.cuh"
+#include "trace64.cuh"
 
 namespace fqsl {
 namespace {
@@ -12,7 +12,7 @@ constexpr int kBlock = 128;
 template <int SRC>
 __global__ void __launch_bounds__(kBlock, FQSL_TRACE_F64_MINB) k_trace_rect_f64(const TraceArgs A)
 {
-    trace::trace_body<double, SRC, true, 0, false, false, true>(A, BatchArgs{});
+    trace64::trace_body<SRC, false, false, true, 0>(A, BatchArgs{});
 }
 // Method II (deviation vectors) on a stretched grid
 template <int WAY>
@@ -25,7 +25,7 @@ __global__ void __launch_bounds__(kBlock) k_trace_dev_rect_f64(const TraceArgs A
 template <int SRC>
 __global__ void __launch_bounds__(kBlock, FQSL_TRACE_F64_MINB) k_trace_tape_rect_f64(const TraceArgs A)
 {
-    trace::trace_body<double, SRC, true, 0, false, true, true>(A, BatchArgs{});
+    trace64::trace_body<SRC, false, true, true, 0>(A, BatchArgs{});
 }
 }  // namespace
 

@@ -2,16 +2,16 @@
 // 2.3; Eq. step) on stretched grids (Sec. 2.2-2.3). Built without
 // contraction like trace_f64.cu, so that it reproduces a plain evaluation of
 // the method to the last bit.
-#include "trace.cuh"
+#include "trace64.cuh"
 
 namespace fqsl {
 namespace {
 constexpr int kBlock = 128;
 
 template <int SRC>
-__global__ void __launch_bounds__(kBlock) k_trace_rect_rk38_f64(const TraceArgs A)
+__global__ void __launch_bounds__(kBlock, FQSL_TRACE_F64_MINB) k_trace_rect_rk38_f64(const TraceArgs A)
 {
-    trace::trace_body<double, SRC, true, 0, false, false, true, 1>(A, BatchArgs{});
+    trace64::trace_body<SRC, false, false, true, 1>(A, BatchArgs{});
 }
 
 template <int WAY>
@@ -22,9 +22,9 @@ __global__ void __launch_bounds__(kBlock) k_trace_dev_rect_rk38_f64(const TraceA
 
 // the adjoint's forward pass: lattice or extra lines writing the step tape
 template <int SRC>
-__global__ void __launch_bounds__(kBlock) k_trace_tape_rect_rk38_f64(const TraceArgs A)
+__global__ void __launch_bounds__(kBlock, FQSL_TRACE_F64_MINB) k_trace_tape_rect_rk38_f64(const TraceArgs A)
 {
-    trace::trace_body<double, SRC, true, 0, false, true, true, 1>(A, BatchArgs{});
+    trace64::trace_body<SRC, false, true, true, 1>(A, BatchArgs{});
 }
 }  // namespace
 

@@ -2,16 +2,16 @@
 // 3/8-rule RK4 with the per-line step of Sec. 4 Eq. step). Built without
 // contraction like trace_f64.cu, so that it reproduces a plain evaluation of
 // the method to the last bit.
-#include "trace.cuh"
+#include "trace64.cuh"
 
 namespace fqsl {
 namespace {
 constexpr int kBlock = 128;
 
 template <int SRC>
-__global__ void __launch_bounds__(kBlock) k_trace_rk38_f64(const TraceArgs A)
+__global__ void __launch_bounds__(kBlock, FQSL_TRACE_F64_MINB) k_trace_rk38_f64(const TraceArgs A)
 {
-    trace::trace_body<double, SRC, true, 0, false, false, false, 1>(A, BatchArgs{});
+    trace64::trace_body<SRC, false, false, false, 1>(A, BatchArgs{});
 }
 
 template <int WAY>
@@ -22,16 +22,16 @@ __global__ void __launch_bounds__(kBlock) k_trace_dev_rk38_f64(const TraceArgs A
 
 // batches: many (field, plane) entries in one launch
 template <int SRC>
-__global__ void __launch_bounds__(kBlock) k_batch_trace_rk38_f64(const TraceArgs A0, const BatchArgs B)
+__global__ void __launch_bounds__(kBlock, FQSL_TRACE_F64_MINB) k_batch_trace_rk38_f64(const TraceArgs A0, const BatchArgs B)
 {
-    trace::trace_body<double, SRC, true, 0, true, false, false, 1>(A0, B);
+    trace64::trace_body<SRC, true, false, false, 1>(A0, B);
 }
 
 // the adjoint's forward pass: lattice or extra lines writing the step tape
 template <int SRC>
-__global__ void __launch_bounds__(kBlock) k_trace_tape_rk38_f64(const TraceArgs A)
+__global__ void __launch_bounds__(kBlock, FQSL_TRACE_F64_MINB) k_trace_tape_rk38_f64(const TraceArgs A)
 {
-    trace::trace_body<double, SRC, true, 0, false, true, false, 1>(A, BatchArgs{});
+    trace64::trace_body<SRC, false, true, false, 1>(A, BatchArgs{});
 }
 }  // namespace
 
