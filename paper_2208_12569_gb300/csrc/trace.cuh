@@ -1153,12 +1153,22 @@ __device__ __forceinline__ void store_state(float *p, float x, float y, float z)
 {
     *(float4 *)p = make_float4(x, y, z, 0.f);
 }
+__device__ __forceinline__ void store_state(double *p, double x, double y, double z)
+{
+    ((double2 *)p)[0] = make_double2(x, y);
+    ((double2 *)p)[1] = make_double2(z, 0.0);
+}
 // the first N (a multiple of 4) values of v
 template <typename T, int N>
 __device__ __forceinline__ void store_vec(T *p, const T v[])
 {
+    if constexpr (sizeof(T) == 4) {
 #pragma unroll
-    for (int q = 0; q < N; q += 4) *(float4 *)(p + q) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
+        for (int q = 0; q < N; q += 4) *(float4 *)(p + q) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
+    } else {
+#pragma unroll
+        for (int q = 0; q < N; q += 2) *(double2 *)(p + q) = make_double2(v[q], v[q + 1]);
+    }
 }
 
 // Open a new chunk whose checkpoint is the current state. Returns false when
