@@ -644,7 +644,10 @@ int tlb_blocks(size_t record_bytes, SeedKind kind, bool sparse, int bps)
 //     500 seeds 0.36 -> 0.26 ms with 2 lanes, plane of 4,096 seeds 0.38 -> 0.32
 //     ms with 4, of 40,000 0.58 -> 0.51 ms with 16; with more warps than fit at
 //     once it loses: 90,000 seeds of a plane 0.62 -> 0.84 ms, a list of 40,604
-//     seeds 0.45 -> 0.56 ms). The FP64 tracer of Method I gives a line eight
+//     seeds 0.45 -> 0.56 ms). Whole lines, one after the other, are spread less
+//     below 16 lanes: 8,000 seeds of a list in a 64x64x64 cube 0.160 ms with 8
+//     lanes and 0.177 with 4, 128x128 seeds of its bottom 0.287 ms with 16, 0.295
+//     with 8 and 0.290 with 32. The FP64 tracer of Method I gives a line eight
 //     lanes, so four lines fill a warp. FP64 Method II lines, one per lane, are
 //     spread only over SMs that would idle: their warp instructions take the
 //     narrow FP64 pipe the same time whatever their lanes.
@@ -663,8 +666,10 @@ Spread spread_of(const fqsl_field f, const fqsl_params *p, int bps, long long li
     const long long items = (r.split ? 2 : 1) * lines;
     const int per = lanes_per_line(p);
     const long long most = !f32 && per == 1 ? f->sms : (f32 && kind == kSeedsFace ? warps + warps / 16 : warps);
+    // below 16 lanes, whole lines wait until they would fill half of the warps only
+    const bool half = f32 && !r.split;
     if (p->chunk_tiles == 0 || per > 1)
-        while (r.lanes > per && items <= most * (r.lanes / per / 2)) r.lanes /= 2;
+        while (r.lanes > per && (half && r.lanes < 32 ? 2 : 1) * items <= most * (r.lanes / per / 2)) r.lanes /= 2;
     return r;
 }
 
