@@ -1110,6 +1110,7 @@ fqsl_status run_qmap_locked(fqsl_field f, const Lattice &lat0, const fqsl_params
     a.p.merge = !tape && f32 && rot && !f->timing;
     if (f32) {
         e = launch_seed_prep_f32(a, n, stream);
+        if (e == cudaSuccess && rot && !tape) e = launch_extra_prep_f32(a, stream);
         if (e != cudaSuccess) return cuda_fail(e, who);
     }
     mark(f, 0, stream);
@@ -1516,6 +1517,7 @@ extern "C" fqsl_status fqsl_qmap_plane_static(fqsl_field f, const double origin[
     a.p.merge = f32 && rot && !f->timing;
     if (f32) {
         e = launch_seed_prep_f32(a, n, stream);
+        if (e == cudaSuccess && rot) e = launch_extra_prep_f32(a, stream);
         if (e != cudaSuccess) return cuda_fail(e, who);
     }
     mark(f, 0, stream);
@@ -1768,6 +1770,7 @@ extern "C" fqsl_status fqsl_batch_run(fqsl_batch b, void *cuda_stream)
     a0.p.merge = f32 && b->any_rot;
     if (a0.p.merge) {
         e = launch_batch_extra_prefix(b->d_rot_counts, b->nent, b->d_xbase, s);
+        if (e == cudaSuccess) e = launch_batch_extra_prep_f32(b->d_desc, b->d_xbase, b->nent, s);
         if (e != cudaSuccess) return cuda_fail(e, who);
     }
     BatchArgs ba{b->d_desc, b->d_ibase, b->nent, b->d_xbase};

@@ -327,6 +327,10 @@ constexpr int kTraceBlock = 128;
 cudaError_t launch_assemble(const AssembleArgs &a, cudaStream_t s);
 cudaError_t launch_assemble_f32(const AssembleArgs &a, cudaStream_t s);
 cudaError_t launch_seed_prep_f32(const TraceArgs &a, long long n, cudaStream_t s);
+// the extra lines of the rotated seeds that the pre-pass queued (DevParams::merge)
+cudaError_t launch_extra_prep_f32(const TraceArgs &a, cudaStream_t s);
+cudaError_t launch_extra_prep_rect_f32(const TraceArgs &a, unsigned grid, cudaStream_t s);
+cudaError_t launch_batch_extra_prep_f32(const TraceArgs *desc, const long long *xbase, int nent, cudaStream_t s);
 
 // batches
 cudaError_t launch_batch_seed_prep_f32(const TraceArgs *desc, const long long *nbase, int nent, long long total,

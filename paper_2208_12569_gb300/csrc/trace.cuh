@@ -1512,6 +1512,67 @@ __device__ __forceinline__ bool start_line(const TraceArgs &A, const LineRecs &R
     return true;
 }
 
+// FP32: a line at (x, y, z) orientated by s0, with tol^2 (or the fixed step) w.
+template <typename T, bool ACC>
+__device__ __forceinline__ void set_line32(const TraceArgs &A, Lane<T> &L, float x, float y, float z, float w, bool neg,
+                                           int st)
+{
+    L.sx = L.x = x;
+    L.sy = L.y = y;
+    L.sz = L.z = z;
+    L.tolf2 = w;
+    L.tol = (double)w;
+    L.s0 = neg ? (T)-1 : (T)1;
+    L.st = st;
+    L.steps = 0;
+    L.end = 0;
+    L.mode = 0;
+    L.tcur = -1;
+    L.tn = 0;
+    acc_reset<T, ACC>(L);
+    L.h = A.p.scheme == 1 ? (T)w : (T)A.p.h0;  // fixed step: the pre-pass's step
+}
+
+// FP32: lattice seed idx from the seed pre-pass, which did the set-up and wrote
+// the final records of seeds outside the box or on a null.
+template <typename T, bool ACC, int DEV = 0>
+__device__ __forceinline__ bool load_seed(const TraceArgs &A, Lane<T> &L, long long idx)
+{
+    L.line = idx;
+    const uint8_t fl = A.prep.flags[idx];
+    if (fl & kSeedDone) return false;
+    const float4 sd = A.prep.seed[idx];
+    set_line32<T, ACC>(A, L, sd.x, sd.y, sd.z, sd.w, (fl & kSeedNegS0) != 0, (fl & kSeedRotated) ? FQSL_LINE_ROTATED : 0);
+    if constexpr (DEV != 0) {
+        const float4 fu = A.prep.fu[idx], fv = A.prep.fv[idx];
+        L.u[0] = L.u0[0] = fu.x;
+        L.u[1] = L.u0[1] = fu.y;
+        L.u[2] = L.u0[2] = fu.z;
+        L.v[0] = L.v0[0] = fv.x;
+        L.v[1] = L.v0[1] = fv.y;
+        L.v[2] = L.v0[2] = fv.z;
+    }
+    return true;
+}
+
+// FP32: record idx of an extra line as extra_prep_f32 left it: its seed in the end
+// records of both directions (each overwritten by that direction's end only),
+// its orientation in the faces (-1: the line is finished).
+template <typename T, bool ACC>
+__device__ __forceinline__ bool load_extra(const TraceArgs &A, Lane<T> &L, long long idx, int dir)
+{
+    const LineRecs &R = A.rec;
+    L.line = idx;
+    const int fl = (dir ? R.f2 : R.f1)[idx];
+    if (fl < 0) return false;
+    const float *r = (dir ? R.xi2 : R.xi1) + 3 * idx;
+    // the perpendicular tolerance, squared in double (as start_line keeps it)
+    const double c = ctl_perp(A.p), tol = A.p.scheme == 1 ? c : c * c;
+    set_line32<T, ACC>(A, L, r[0], r[1], r[2], (float)tol, fl != 0, 0);
+    L.tol = tol;
+    return true;
+}
+
 // Lattice seed: frame, tolerance and rotation decision (Sec. 4). reg_rot:
 // queue a rotated seed for its extra lines (once per seed).
 template <typename T, bool ACC, int DEV = 0, bool RECT = false>
@@ -1533,37 +1594,7 @@ __device__ __forceinline__ bool init_lattice(const TraceArgs &A, Lane<T> &L, lon
     L.line = idx;
     const FieldView &f = A.f;
     const LineRecs &R = A.rec;
-    if constexpr (!kF64) {
-        // FP32: the seed pre-pass did the set-up (and wrote final records of
-        // seeds outside the box or on a null)
-        const uint8_t fl = A.prep.flags[idx];
-        if (fl & kSeedDone) return false;
-        const float4 sd = A.prep.seed[idx];
-        L.sx = L.x = sd.x;
-        L.sy = L.y = sd.y;
-        L.sz = L.z = sd.z;
-        L.tolf2 = sd.w;
-        L.tol = (double)sd.w;
-        L.s0 = (fl & kSeedNegS0) ? (T)-1 : (T)1;
-        L.st = (fl & kSeedRotated) ? FQSL_LINE_ROTATED : 0;
-        L.steps = 0;
-        L.end = 0;
-        L.mode = 0;
-        L.tcur = -1;
-        L.tn = 0;
-        acc_reset<T, ACC>(L);
-        L.h = A.p.scheme == 1 ? (T)sd.w : (T)A.p.h0;  // fixed step: the pre-pass's step
-        if constexpr (DEV != 0) {
-            const float4 fu = A.prep.fu[idx], fv = A.prep.fv[idx];
-            L.u[0] = L.u0[0] = fu.x;
-            L.u[1] = L.u0[1] = fu.y;
-            L.u[2] = L.u0[2] = fu.z;
-            L.v[0] = L.v0[0] = fv.x;
-            L.v[1] = L.v0[1] = fv.y;
-            L.v[2] = L.v0[2] = fv.z;
-        }
-        return true;
-    }
+    if constexpr (!kF64) return load_seed<T, ACC, DEV>(A, L, idx);
     double xi[3];
     if (kF64) {
         // physical seed, then (r0 - o)/d, as written (the physical seed itself
@@ -1807,7 +1838,9 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A0, const BatchArgs 
                         } else if constexpr (MERGED) {
                             const long long x = slot - nlat - ck_base;
                             fl |= kLaneExtra;
-                            active = x < 4LL * (long long)*E.q.rot_count && init_extra<T, ACC, RECT, true>(E, L, x);
+                            active = x < 4LL * (long long)*E.q.rot_count &&
+                                     load_extra<T, ACC>(E, L, E.lat.n1 * E.lat.n2 * E.lat.n3 + x,
+                                                        psplit ? (int)(item >> 5) & 1 : 0);
                         }
                         if (FLEX && active) {
                             L.st |= fl;
@@ -2275,6 +2308,19 @@ __device__ __forceinline__ void seed_prep_f32(const TraceArgs &A, long long idx)
     // w: tol^2, or with the fixed-step scheme the line's step
     A.prep.seed[idx] = make_float4(x, y, z, A.p.scheme == 1 ? (float)tol : (float)(tol * tol));
     A.prep.flags[idx] = fl;
+}
+
+// FP32 set-up of extra line x (4 slot + q) of a rotated seed, one thread each, for
+// load_extra. (In the tracer it took the registers of the hot loop: a lattice
+// kernel with it ran 10 % slower than one without, 17 % on some sizes.)
+template <bool RECT = false>
+__device__ __forceinline__ void extra_prep_f32(const TraceArgs &A, long long x)
+{
+    Lane<float> L;
+    if (!init_extra<float, false, RECT, true>(A, L, x)) return;  // its final record is written, faces -1
+    const int fl = L.s0 < 0.f ? 1 : 0;
+    write_end32(A.rec, L.line, 0, L.sx, L.sy, L.sz, fl);
+    write_end32(A.rec, L.line, 1, L.sx, L.sy, L.sz, fl);
 }
 
 }  // namespace trace

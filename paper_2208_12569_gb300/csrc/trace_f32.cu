@@ -92,6 +92,55 @@ cudaError_t launch_seed_prep_f32(const TraceArgs &a, long long n, cudaStream_t s
 
 namespace fqsl {
 namespace {
+__global__ void __launch_bounds__(128) k_extra_prep_f32(const TraceArgs A)
+{
+    const long long m = 4LL * (long long)*A.q.rot_count;
+    for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < m; x += (long long)gridDim.x * blockDim.x)
+        trace::extra_prep_f32(A, x);
+}
+
+__global__ void __launch_bounds__(128) k_batch_extra_prep_f32(const TraceArgs *__restrict__ desc,
+                                                              const long long *__restrict__ xbase, int nent)
+{
+    const long long total = xbase[nent];
+    for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < total;
+         x += (long long)gridDim.x * blockDim.x) {
+        int lo = 0, hi = nent - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (xbase[mid] <= x) lo = mid;
+            else hi = mid - 1;
+        }
+        if (x - xbase[lo] < 4LL * (long long)*desc[lo].q.rot_count) trace::extra_prep_f32(desc[lo], x - xbase[lo]);
+    }
+}
+
+unsigned sm_grid(int per_sm)
+{
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return (unsigned)(sms * per_sm);
+}
+}  // namespace
+
+cudaError_t launch_extra_prep_f32(const TraceArgs &a, cudaStream_t s)
+{
+    if (a.f.rect) return launch_extra_prep_rect_f32(a, sm_grid(4), s);
+    k_extra_prep_f32<<<sm_grid(4), 128, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_batch_extra_prep_f32(const TraceArgs *desc, const long long *xbase, int nent, cudaStream_t s)
+{
+    k_batch_extra_prep_f32<<<sm_grid(4), 128, 0, s>>>(desc, xbase, nent);
+    return cudaGetLastError();
+}
+
+}  // namespace fqsl
+
+namespace fqsl {
+namespace {
 template <int WAY, bool FLEX>
 __global__ void __launch_bounds__(kBlock, FQSL_TRACE_DEV_F32_MINB) k_trace_dev_f32(const TraceArgs A)
 {

@@ -120,6 +120,21 @@ int trace_tape_rect_blocks_per_sm_f32(int src, bool acc64)
     return b > 0 ? b : 1;
 }
 
+namespace {
+__global__ void __launch_bounds__(128) k_extra_prep_rect_f32(const TraceArgs A)
+{
+    const long long m = 4LL * (long long)*A.q.rot_count;
+    for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < m; x += (long long)gridDim.x * blockDim.x)
+        trace::extra_prep_f32<true>(A, x);
+}
+}  // namespace
+
+cudaError_t launch_extra_prep_rect_f32(const TraceArgs &a, unsigned grid, cudaStream_t s)
+{
+    k_extra_prep_rect_f32<<<grid, 128, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_seed_prep_rect_f32(const TraceArgs &a, long long n, unsigned grid, cudaStream_t s)
 {
     k_seed_prep_rect_f32<<<grid, 256, 0, s>>>(a, n);
