@@ -673,6 +673,16 @@ Spread spread_of(const fqsl_field f, const fqsl_params *p, int bps, long long li
     return r;
 }
 
+// Lanes of a warp that take lines in a taped launch of `items` directions.
+int tape_lanes(const fqsl_params *p, long long warps, long long items)
+{
+    const int per = lanes_per_line(p);
+    int lanes = 32;
+    if (p->chunk_tiles == 0 || per > 1)
+        while (lanes > per && items <= warps * (lanes / per / 2)) lanes /= 2;
+    return lanes;
+}
+
 // Are a lattice's seeds a cell or more apart (its 8x4-seed tile covers at
 // least as many cells as it has seeds)?
 bool sparse_lattice(const FieldView &g, const Lattice &lat)
@@ -1140,8 +1150,10 @@ fqsl_status run_qmap_locked(fqsl_field f, const Lattice &lat0, const fqsl_params
         long long grid = (long long)f->sms * bps;
         a.nitems *= 2;  // one item per direction of a line
         const int per = lanes_per_line(p);
-        if (per > 1) a.p.chunk = 32 / per;
-        const long long need = (a.nitems * per + kTraceBlock - 1) / kTraceBlock;
+        // (of a face plane's directions half end at once)
+        a.p.lanes = tape_lanes(p, (long long)f->sms * bps * (kTraceBlock / 32), face_plane ? n : 2 * n);
+        if (per > 1 || a.p.lanes < 32) a.p.chunk = a.p.lanes / per;
+        const long long need = (a.nitems * (32 / a.p.lanes) * per + kTraceBlock - 1) / kTraceBlock;
         if (need < grid) grid = need;
         if (grid < 1) grid = 1;
         e = launch_tape(a, p, kSrcLattice, grid, stream);
@@ -1156,6 +1168,8 @@ fqsl_status run_qmap_locked(fqsl_field f, const Lattice &lat0, const fqsl_params
             // their count is read on the device (persistent grid)
             a.q.head = tl.ctr + 5;
             a.tape.hl_base = 2 * n;
+            a.p.lanes = 32;
+            a.p.chunk = 32 / lanes_per_line(p);
             int bps = tape_blocks_per_sm(f, p->precision, kSrcExtra, p->scheme);
             if (p->blocks_per_sm > 0 && p->blocks_per_sm < bps) bps = p->blocks_per_sm;
             e = launch_tape(a, p, kSrcExtra, (long long)f->sms * bps, stream);

@@ -1910,77 +1910,85 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A0, const BatchArgs 
         T l4 = 0, tw4 = 0;
         int fail = 0;  // first failing stage: 1 null field, 2 grazing exit step
         constexpr int NST = Tab<T, SCH>::N;
+        // RKF45: an exit step of length 0 (a seed on the face that its direction
+        // leaves by: every line of a face plane has one) evaluates the same point
+        // at every stage, so the first stage's values serve all of them: 128x128
+        // seeds of a 64x64x64 cube 291 -> 282 us. (Not the 3/8 rule: 79,000
+        // seeds 780 us with it, 740 without.)
+        const bool still = SCH == 0 && henon && hh == (T)0;
+        T o[NS];
 #pragma unroll
         for (int s = 0; s < NST; s++) {
-            T px = 0, py = 0, pz = 0;
+            if (s == 0 || !still) {
+                T px = 0, py = 0, pz = 0;
 #pragma unroll
-            for (int r = 0; r < s; r++) {
-                const T c = Tab<T, SCH>::a(s, r);
-                px += c * k0[r];
-                py += c * k1[r];
-                pz += c * k2[r];
-            }
-            px = L.x + hh * px;
-            py = L.y + hh * py;
-            pz = L.z + hh * pz;
-            T o[NS];
-            // FP32: RKF45's stages 1 and 5 have zero 4th-order weight, so their
-            // Tw integrand is not formed (nor their curl B loaded)
-            const bool wj = kF64 || SCH != 0 || (s != 1 && s != 5);
-            Near32 near;  // FP32 Method II way 2: what this evaluation read
-            bool ok = rhsg<RECT>(f, dd, sgn, px, py, pz, o, (RECT && s == 0) ? &rc0 : nullptr, wj,
-                                 (DEV == 2 && !kF64) ? &near : nullptr);
-            if constexpr (DEV != 0) {
-                // stage deviation vectors and Eq. rb2: dU/dtau = sigma (ds/dtau) (U . grad)(B/|B|)
-                T us[6];
-#pragma unroll
-                for (int c = 0; c < 6; c++) {
-                    T acc = 0;
-#pragma unroll
-                    for (int r = 0; r < s; r++) acc += Tab<T, SCH>::a(s, r) * kd[r][c];
-                    us[c] = (c < 3 ? L.u[c] : L.v[c - 3]) + hh * acc;
+                for (int r = 0; r < s; r++) {
+                    const T c = Tab<T, SCH>::a(s, r);
+                    px += c * k0[r];
+                    py += c * k1[r];
+                    pz += c * k2[r];
                 }
-                const T sdl = sgn * o[3];
-                if constexpr (DEV == 2 && !kF64) {
-                    float su[3], sv[3];
-                    ok = grad_way2_32<RECT>(f, (float)A0.p.eps2, px, py, pz, dd, near, us, su, sv) && ok;
+                px = L.x + hh * px;
+                py = L.y + hh * py;
+                pz = L.z + hh * pz;
+                // FP32: RKF45's stages 1 and 5 have zero 4th-order weight, so their
+                // Tw integrand is not formed (nor their curl B loaded)
+                const bool wj = kF64 || SCH != 0 || (s != 1 && s != 5);
+                Near32 near;  // FP32 Method II way 2: what this evaluation read
+                bool ok = rhsg<RECT>(f, dd, sgn, px, py, pz, o, (RECT && s == 0) ? &rc0 : nullptr, wj,
+                                     (DEV == 2 && !kF64) ? &near : nullptr);
+                if constexpr (DEV != 0) {
+                    // stage deviation vectors and Eq. rb2: dU/dtau = sigma (ds/dtau) (U . grad)(B/|B|)
+                    T us[6];
 #pragma unroll
-                    for (int b = 0; b < 3; b++) {
-                        o[5 + b] = sdl * su[b];
-                        o[8 + b] = sdl * sv[b];
+                    for (int c = 0; c < 6; c++) {
+                        T acc = 0;
+#pragma unroll
+                        for (int r = 0; r < s; r++) acc += Tab<T, SCH>::a(s, r) * kd[r][c];
+                        us[c] = (c < 3 ? L.u[c] : L.v[c - 3]) + hh * acc;
                     }
-                } else {
-                    T G[3][3];
-                    ok = grad_bhat<T, DEV, RECT>(f, (T)A0.p.eps2, px, py, pz, dd, G) && ok;
+                    const T sdl = sgn * o[3];
+                    if constexpr (DEV == 2 && !kF64) {
+                        float su[3], sv[3];
+                        ok = grad_way2_32<RECT>(f, (float)A0.p.eps2, px, py, pz, dd, near, us, su, sv) && ok;
 #pragma unroll
-                    for (int b = 0; b < 3; b++) {
-                        T su = 0, sv = 0;
-#pragma unroll
-                        for (int a = 0; a < 3; a++) {
-                            su += us[a] * G[a][b];
-                            sv += us[3 + a] * G[a][b];
+                        for (int b = 0; b < 3; b++) {
+                            o[5 + b] = sdl * su[b];
+                            o[8 + b] = sdl * sv[b];
                         }
-                        o[5 + b] = sdl * su;
-                        o[8 + b] = sdl * sv;
+                    } else {
+                        T G[3][3];
+                        ok = grad_bhat<T, DEV, RECT>(f, (T)A0.p.eps2, px, py, pz, dd, G) && ok;
+#pragma unroll
+                        for (int b = 0; b < 3; b++) {
+                            T su = 0, sv = 0;
+#pragma unroll
+                            for (int a = 0; a < 3; a++) {
+                                su += us[a] * G[a][b];
+                                sv += us[3 + a] * G[a][b];
+                            }
+                            o[5 + b] = sdl * su;
+                            o[8 + b] = sdl * sv;
+                        }
                     }
                 }
-            }
-            if (!ok && !fail) fail = 1;
-            if (henon) {
-                const T fa = sel3<T>(hax, o[0], o[1], o[2]);
-                // grazing test in cells per unit tau (physical velocity over the cell width)
-                T fn = fa;
-                if constexpr (RECT) fn = kF64 ? fa / sel3<T>(hax, dd[0], dd[1], dd[2]) : fa * sel3<T>(hax, dd[0], dd[1], dd[2]);
-                const bool bad = !(fn * hsign >= graze);
-                if (bad && !fail) fail = 2;
-                if (kF64) {
-                    const T den = bad ? (T)1 : fa;
+                if (!ok && !fail) fail = 1;
+                if (henon) {
+                    const T fa = sel3<T>(hax, o[0], o[1], o[2]);
+                    // grazing test in cells per unit tau (physical velocity over the cell width)
+                    T fn = fa;
+                    if constexpr (RECT) fn = kF64 ? fa / sel3<T>(hax, dd[0], dd[1], dd[2]) : fa * sel3<T>(hax, dd[0], dd[1], dd[2]);
+                    const bool bad = !(fn * hsign >= graze);
+                    if (bad && !fail) fail = 2;
+                    if (kF64) {
+                        const T den = bad ? (T)1 : fa;
 #pragma unroll
-                    for (int c = 0; c < NS; c++) o[c] = o[c] / den;
-                } else {
-                    const T inv = bad ? (T)0 : (T)1 / fa;
+                        for (int c = 0; c < NS; c++) o[c] = o[c] / den;
+                    } else {
+                        const T inv = bad ? (T)0 : (T)1 / fa;
 #pragma unroll
-                    for (int c = 0; c < NS; c++) o[c] *= inv;
+                        for (int c = 0; c < NS; c++) o[c] *= inv;
+                    }
                 }
             }
             // (the 3/8 rule's last stage is kept too when the tape holds the

@@ -679,9 +679,12 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A0, const BatchArgs 
         double ws = 0.0;
         const int own = g.sub < 5 ? g.sub : g.sub - 5;
         int fail = 0;  // first failing stage: 1 null field, 2 grazing exit step
+        // (an exit step of length 0 evaluates one point: see trace.cuh)
+        const bool still = henon && hh == 0.0;
+        double o = 0.0;
 #pragma unroll 1
         for (int s = 0; s < NST; s++) {
-            if (s > 0) {
+            if (s > 0 && !still) {
                 // sum of a(s, r) k_r over r, left to right; lanes 0-2 form the
                 // products of even r, lanes 4-6 those of the odd r behind them
                 double p = 0.0;
@@ -696,15 +699,17 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A0, const BatchArgs 
                 if (g.a == 3) x = 0.0;
                 cx = cell_of<RECT>(ax, g, x, wx, width);
             }
-            double o = 0.0;
-            const bool ok = rhs<RECT>(f, g, cx, wx, dD, sgn, o);
-            if (!ok && !fail) fail = 1;
-            if (henon) {
-                const double fa = get(g, o, hax);
-                const double fn = RECT ? div64(fa, get(g, D, hax)) : fa;
-                const bool bad = !(turn(hsign, fn) >= graze);
-                if (bad && !fail) fail = 2;
-                o = div64(o, bad ? 1.0 : fa);
+            if (s == 0 || !still) {
+                o = 0.0;
+                const bool ok = rhs<RECT>(f, g, cx, wx, dD, sgn, o);
+                if (!ok && !fail) fail = 1;
+                if (henon) {
+                    const double fa = get(g, o, hax);
+                    const double fn = RECT ? div64(fa, get(g, D, hax)) : fa;
+                    const bool bad = !(turn(hsign, fn) >= graze);
+                    if (bad && !fail) fail = 2;
+                    o = div64(o, bad ? 1.0 : fa);
+                }
             }
             const double ka = get(g, o, g.a);
             if (s < 5) k[s] = ka;
