@@ -11,20 +11,24 @@
 // non-uniform axis are used, in FP64. One thread per node, grid-stride;
 // streaming and HBM-bound.
 #include "fqsl_internal.cuh"
+#include "soft64.cuh"
 
 namespace fqsl {
 namespace {
 
 template <typename TI>
 __device__ __forceinline__ double node_diff(const TI *__restrict__ B, int c, long long node, long long stride,
-                                            long long i, long long n, double h)
+                                            long long i, long long n, const soft64::Divisor &h)
 {
-    // value of component c at index kk along the axis (node is at index i)
+    // value of component c at index kk along the axis (node is at index i);
+    // h: the spacing (2 nodes) or twice it
     auto F = [&](long long kk) -> double { return (double)B[(node + (kk - i) * stride) * 3 + c]; };
-    if (n == 2) return (F(1) - F(0)) / h;
-    if (i == 0) return (-3.0 * F(0) + 4.0 * F(1) - F(2)) / (2.0 * h);
-    if (i == n - 1) return (3.0 * F(n - 1) - 4.0 * F(n - 2) + F(n - 3)) / (2.0 * h);
-    return (F(i + 1) - F(i - 1)) / (2.0 * h);
+    double v;
+    if (n == 2) v = F(1) - F(0);
+    else if (i == 0) v = -3.0 * F(0) + 4.0 * F(1) - F(2);
+    else if (i == n - 1) v = 3.0 * F(n - 1) - 4.0 * F(n - 2) + F(n - 3);
+    else v = F(i + 1) - F(i - 1);
+    return soft64::div64(v, h);
 }
 
 template <typename TI>
@@ -34,17 +38,22 @@ __global__ void __launch_bounds__(256) k_curl_pack(const TI *__restrict__ B, int
 {
     const long long total = (long long)nx * ny * nz;
     const long long sy = nx, sz = (long long)nx * ny;
+    // the six divisions of a node run on the integer pipe (same bits): they held
+    // the FP64 pipe for about 60 of the node's 75 instructions (FP64 records of
+    // 256x256x128 nodes of an FP64 cube 1.09 -> 0.62 ms)
+    const soft64::Divisor hx = soft64::divisor(nx == 2 ? dx : 2.0 * dx), hy = soft64::divisor(ny == 2 ? dy : 2.0 * dy),
+                          hz = soft64::divisor(nz == 2 ? dz : 2.0 * dz);
     for (long long node = blockIdx.x * (long long)blockDim.x + threadIdx.x; node < total;
          node += (long long)gridDim.x * blockDim.x) {
         const long long i = node % nx;
         const long long j = (node / nx) % ny;
         const long long k = node / sz;
-        const double dyBz = node_diff(B, 2, node, sy, j, ny, dy);
-        const double dzBy = node_diff(B, 1, node, sz, k, nz, dz);
-        const double dzBx = node_diff(B, 0, node, sz, k, nz, dz);
-        const double dxBz = node_diff(B, 2, node, 1, i, nx, dx);
-        const double dxBy = node_diff(B, 1, node, 1, i, nx, dx);
-        const double dyBx = node_diff(B, 0, node, sy, j, ny, dy);
+        const double dyBz = node_diff(B, 2, node, sy, j, ny, hy);
+        const double dzBy = node_diff(B, 1, node, sz, k, nz, hz);
+        const double dzBx = node_diff(B, 0, node, sz, k, nz, hz);
+        const double dxBz = node_diff(B, 2, node, 1, i, nx, hx);
+        const double dxBy = node_diff(B, 1, node, 1, i, nx, hx);
+        const double dyBx = node_diff(B, 0, node, sy, j, ny, hy);
         const double Jx = dyBz - dzBy, Jy = dzBx - dxBz, Jz = dxBy - dyBx;
         const double Bx = (double)B[node * 3 + 0], By = (double)B[node * 3 + 1], Bz = (double)B[node * 3 + 2];
         if (rec32) {
@@ -148,85 +157,124 @@ __global__ void __launch_bounds__(256) k_curl_pack32(const float *__restrict__ B
     }
 }
 
-// Component c of B/|B| at a node (0 where |B| = 0), as written.
+// B/|B| at a node (0 where |B| = 0), the divisions and the root on the integer
+// pipe (soft64.cuh; same bits).
+struct Unit {
+    double v[3];
+};
+
 template <typename TI>
-__device__ __forceinline__ double bhat(const TI *__restrict__ B, long long q, int c)
+__device__ __forceinline__ Unit bhat(const TI *__restrict__ B, long long q)
 {
     const double b0 = (double)B[3 * q], b1 = (double)B[3 * q + 1], b2 = (double)B[3 * q + 2];
-    const double m = sqrt(b0 * b0 + b1 * b1 + b2 * b2);
-    const double bc = c == 0 ? b0 : (c == 1 ? b1 : b2);
-    return m > 0 ? bc / m : 0.0;
-}
-
-template <typename TI>
-__device__ __forceinline__ double bhat_diff(const TI *__restrict__ B, int c, long long node, long long stride,
-                                            long long i, long long n, double h)
-{
-    auto F = [&](long long kk) -> double { return bhat(B, node + (kk - i) * stride, c); };
-    if (n == 2) return (F(1) - F(0)) / h;
-    if (i == 0) return (-3.0 * F(0) + 4.0 * F(1) - F(2)) / (2.0 * h);
-    if (i == n - 1) return (3.0 * F(n - 1) - 4.0 * F(n - 2) + F(n - 3)) / (2.0 * h);
-    return (F(i + 1) - F(i - 1)) / (2.0 * h);
-}
-
-// Stretched grid: the same with the three-point stencils of node_diff_rect
-template <typename TI>
-__device__ __forceinline__ double bhat_diff_rect(const TI *__restrict__ B, int c, long long node, long long stride,
-                                                 long long i, long long n, const double *__restrict__ X,
-                                                 const double *__restrict__ co)
-{
-    auto F = [&](long long kk) -> double { return bhat(B, node + (kk - i) * stride, c); };
-    if (n == 2) return (F(1) - F(0)) / (X[1] - X[0]);
-    const double c0 = co[3 * i], c1 = co[3 * i + 1], c2 = co[3 * i + 2];
-    if (i == 0) return c0 * F(0) + c1 * F(1) - c2 * F(2);
-    if (i == n - 1) return c0 * F(n - 3) - c1 * F(n - 2) + c2 * F(n - 1);
-    return c0 * F(i - 1) + c1 * F(i) + c2 * F(i + 1);
-}
-
-template <typename TI>
-__global__ void __launch_bounds__(256) k_gradb_pack_rect(const TI *__restrict__ B, const FieldView g,
-                                                         float *__restrict__ g32, double *__restrict__ g64)
-{
-    const long long nx = g.nx, ny = g.ny, nz = g.nz;
-    const long long total = nx * ny * nz;
-    const long long stride[3] = {1, nx, nx * ny};
-    const long long n[3] = {nx, ny, nz};
-    for (long long node = blockIdx.x * (long long)blockDim.x + threadIdx.x; node < total;
-         node += (long long)gridDim.x * blockDim.x) {
-        const long long idx[3] = {node % nx, (node / nx) % ny, node / stride[2]};
-        for (int a = 0; a < 3; a++)
-            for (int b = 0; b < 3; b++) {
-                const double v = bhat_diff_rect(B, b, node, stride[a], idx[a], n[a], g.x64[a], g.dco[a]);
-                if (g64) g64[node * 10 + a * 3 + b] = v;
-                if (g32) g32[node * 12 + a * 3 + b] = (float)v;
-            }
-        if (g64) g64[node * 10 + 9] = 0.0;
-        if (g32) g32[node * 12 + 9] = g32[node * 12 + 10] = g32[node * 12 + 11] = 0.f;
-    }
+    const double m = soft64::sqrt64(b0 * b0 + b1 * b1 + b2 * b2);
+    const soft64::Divisor d = soft64::divisor(m);
+    Unit u;
+    u.v[0] = m > 0 ? soft64::div64(b0, d) : 0.0;
+    u.v[1] = m > 0 ? soft64::div64(b1, d) : 0.0;
+    u.v[2] = m > 0 ? soft64::div64(b2, d) : 0.0;
+    return u;
 }
 
 // grad(B/|B|) at the nodes for Method II way 1 (Sec. 4, Eq. grad_B): G[a*3+b]
-// = d(B_b/|B|)/dx_a with the stencils of the curl grid.
-template <typename TI>
-__global__ void __launch_bounds__(256) k_gradb_pack(const TI *__restrict__ B, int nx, int ny, int nz, double dx,
-                                                    double dy, double dz, float *__restrict__ g32,
-                                                    double *__restrict__ g64)
+// = d(B_b/|B|)/dx_a with the stencils of the curl grid (RECT: node_diff_rect's).
+// A block holds B/|B| of a tile of 16 x 8 x 4 nodes and its one-node halo in
+// shared memory, so that a node's is formed about twice and not 18 times (its
+// root and divisions are what the kernel spends its time on: repacking 256x256x128
+// nodes with the gradient took 9.54 ms when a thread formed all of a node's
+// differences from B, and takes 1.54 ms); the one-sided differences on the
+// faces, which reach two nodes, form theirs.
+constexpr int kGx = 16, kGy = 8, kGz = 4;
+
+template <typename TI, bool RECT>
+__global__ void __launch_bounds__(kGx *kGy) k_gradb_pack(const TI *__restrict__ B, const FieldView g,
+                                                         float4 *__restrict__ g32, double *__restrict__ g64)
 {
-    const long long total = (long long)nx * ny * nz;
+    __shared__ double U[3][kGz + 2][kGy + 2][kGx + 2];
+    const int nx = g.nx, ny = g.ny, nz = g.nz;
     const long long stride[3] = {1, nx, (long long)nx * ny};
-    const double d[3] = {dx, dy, dz};
-    const long long n[3] = {nx, ny, nz};
-    for (long long node = blockIdx.x * (long long)blockDim.x + threadIdx.x; node < total;
-         node += (long long)gridDim.x * blockDim.x) {
-        const long long idx[3] = {node % nx, (node / nx) % ny, node / stride[2]};
-        for (int a = 0; a < 3; a++)
-            for (int b = 0; b < 3; b++) {
-                const double g = bhat_diff(B, b, node, stride[a], idx[a], n[a], d[a]);
-                if (g64) g64[node * 10 + a * 3 + b] = g;
-                if (g32) g32[node * 12 + a * 3 + b] = (float)g;
+    const int n[3] = {nx, ny, nz};
+    const int tx = (nx + kGx - 1) / kGx, ty = (ny + kGy - 1) / kGy;
+    const long long tiles = (long long)tx * ty * ((nz + kGz - 1) / kGz);
+    for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
+        const int x0 = (int)(t % tx) * kGx, y0 = (int)(t / tx % ty) * kGy, z0 = (int)(t / ((long long)tx * ty)) * kGz;
+        __syncthreads();
+        for (int q = threadIdx.x; q < (kGz + 2) * (kGy + 2) * (kGx + 2); q += kGx * kGy) {
+            const int i = q % (kGx + 2), j = q / (kGx + 2) % (kGy + 2), k = q / ((kGx + 2) * (kGy + 2));
+            const int x = x0 + i - 1, y = y0 + j - 1, z = z0 + k - 1;
+            if (x < 0 || y < 0 || z < 0 || x >= nx || y >= ny || z >= nz) continue;
+            const Unit u = bhat(B, x + nx * (y + (long long)ny * z));
+#pragma unroll
+            for (int c = 0; c < 3; c++) U[c][k][j][i] = u.v[c];
+        }
+        __syncthreads();
+        const int i = threadIdx.x % kGx, j = threadIdx.x / kGx;
+        if (x0 + i >= nx || y0 + j >= ny) continue;
+#pragma unroll 1
+        for (int k = 0; k < kGz && z0 + k < nz; k++) {
+            const int at[3] = {x0 + i, y0 + j, z0 + k};
+            const long long node = at[0] + nx * (at[1] + (long long)ny * at[2]);
+            double G[3][3];
+#pragma unroll
+            for (int a = 0; a < 3; a++) {
+                const int p = at[a], m = n[a];
+                const bool inner = m > 2 && p > 0 && p < m - 1;
+                // B/|B| at the three nodes of the stencil, in its order
+                Unit f[3];
+                if (inner) {
+#pragma unroll
+                    for (int c = 0; c < 3; c++) {
+                        f[0].v[c] = U[c][k + 1 - (a == 2)][j + 1 - (a == 1)][i + 1 - (a == 0)];
+                        f[1].v[c] = U[c][k + 1][j + 1][i + 1];
+                        f[2].v[c] = U[c][k + 1 + (a == 2)][j + 1 + (a == 1)][i + 1 + (a == 0)];
+                    }
+                } else {
+#pragma unroll 1
+                    for (int r = 0; r < 3; r++) {
+                        // first node: 0, 1, 2; last: n - 1, n - 2, n - 3; two nodes: 0, 1
+                        const int q = m == 2 ? min(r, 1) : (p == 0 ? r : m - 1 - r);
+                        const Unit u = bhat(B, node + (long long)(q - p) * stride[a]);
+                        if (r == 0) f[0] = u;
+                        else if (r == 1) f[1] = u;
+                        else f[2] = u;
+                    }
+                }
+                if constexpr (RECT) {
+                    const double *X = g.x64[a], *co = g.dco[a] + 3 * p;
+                    const soft64::Divisor w = soft64::divisor(m == 2 ? X[1] - X[0] : 1.0);
+#pragma unroll
+                    for (int b = 0; b < 3; b++) {
+                        const double f0 = f[0].v[b], f1 = f[1].v[b], f2 = f[2].v[b];
+                        if (m == 2) G[a][b] = soft64::div64(f1 - f0, w);
+                        else if (p == 0) G[a][b] = co[0] * f0 + co[1] * f1 - co[2] * f2;
+                        else if (p == m - 1) G[a][b] = co[0] * f2 - co[1] * f1 + co[2] * f0;
+                        else G[a][b] = co[0] * f0 + co[1] * f1 + co[2] * f2;
+                    }
+                } else {
+                    const soft64::Divisor w = soft64::divisor(m == 2 ? g.d[a] : 2.0 * g.d[a]);
+#pragma unroll
+                    for (int b = 0; b < 3; b++) {
+                        const double f0 = f[0].v[b], f1 = f[1].v[b], f2 = f[2].v[b];
+                        double v;
+                        if (m == 2) v = f1 - f0;
+                        else if (p == 0) v = -3.0 * f0 + 4.0 * f1 - f2;
+                        else if (p == m - 1) v = 3.0 * f0 - 4.0 * f1 + f2;
+                        else v = f2 - f0;
+                        G[a][b] = soft64::div64(v, w);
+                    }
+                }
             }
-        if (g64) g64[node * 10 + 9] = 0.0;
-        if (g32) g32[node * 12 + 9] = g32[node * 12 + 10] = g32[node * 12 + 11] = 0.f;
+            if (g64) {
+#pragma unroll
+                for (int c = 0; c < 9; c++) g64[node * 10 + c] = G[c / 3][c % 3];
+                g64[node * 10 + 9] = 0.0;
+            }
+            if (g32) {
+                g32[3 * node + 0] = make_float4((float)G[0][0], (float)G[0][1], (float)G[0][2], (float)G[1][0]);
+                g32[3 * node + 1] = make_float4((float)G[1][1], (float)G[1][2], (float)G[2][0], (float)G[2][1]);
+                g32[3 * node + 2] = make_float4((float)G[2][2], 0.f, 0.f, 0.f);
+            }
+        }
     }
 }
 
@@ -238,25 +286,14 @@ cudaError_t launch_gradb_pack(const void *B, fqsl_dtype bt, const FieldView &g, 
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const long long total = (long long)g.nx * g.ny * g.nz;
-    long long blocks = (total + 255) / 256;
-    if (blocks > (long long)sms * 8) blocks = (long long)sms * 8;
-    if (blocks < 1) blocks = 1;
-    if (g.rect) {
-        if (bt == FQSL_F32)
-            k_gradb_pack_rect<float><<<(unsigned)blocks, 256, 0, s>>>((const float *)B, g, (float *)grad32,
-                                                                     (double *)grad64);
-        else
-            k_gradb_pack_rect<double><<<(unsigned)blocks, 256, 0, s>>>((const double *)B, g, (float *)grad32,
-                                                                      (double *)grad64);
-        return cudaGetLastError();
-    }
-    if (bt == FQSL_F32)
-        k_gradb_pack<float><<<(unsigned)blocks, 256, 0, s>>>((const float *)B, g.nx, g.ny, g.nz, g.d[0], g.d[1],
-                                                            g.d[2], (float *)grad32, (double *)grad64);
-    else
-        k_gradb_pack<double><<<(unsigned)blocks, 256, 0, s>>>((const double *)B, g.nx, g.ny, g.nz, g.d[0], g.d[1],
-                                                             g.d[2], (float *)grad32, (double *)grad64);
+    const long long tiles = (long long)((g.nx + kGx - 1) / kGx) * ((g.ny + kGy - 1) / kGy) * ((g.nz + kGz - 1) / kGz);
+    const unsigned blocks = (unsigned)(tiles < (long long)sms * 32 ? tiles : (long long)sms * 32);
+    float4 *o32 = (float4 *)grad32;
+    double *o64 = (double *)grad64;
+    if (bt == FQSL_F32 && g.rect) k_gradb_pack<float, true><<<blocks, kGx * kGy, 0, s>>>((const float *)B, g, o32, o64);
+    else if (bt == FQSL_F32) k_gradb_pack<float, false><<<blocks, kGx * kGy, 0, s>>>((const float *)B, g, o32, o64);
+    else if (g.rect) k_gradb_pack<double, true><<<blocks, kGx * kGy, 0, s>>>((const double *)B, g, o32, o64);
+    else k_gradb_pack<double, false><<<blocks, kGx * kGy, 0, s>>>((const double *)B, g, o32, o64);
     return cudaGetLastError();
 }
 
