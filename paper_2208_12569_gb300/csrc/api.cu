@@ -642,9 +642,8 @@ int tlb_blocks(size_t record_bytes, SeedKind kind, bool sparse, int bps)
 //   lanes: fewer lines per warp until the lines fill the resident warps: lanes
 //     of one warp whose lines have parted wait for each other's loads (list of
 //     500 seeds 0.36 -> 0.26 ms with 2 lanes, plane of 4,096 seeds 0.38 -> 0.32
-//     ms with 4, of 40,000 0.58 -> 0.51 ms with 16; with more warps than fit at
-//     once it loses: 90,000 seeds of a plane 0.62 -> 0.84 ms, a list of 40,604
-//     seeds 0.45 -> 0.56 ms). Whole lines, one after the other, are spread less
+//     ms with 4; with more warps than fit at once it loses: 90,000 seeds of a
+//     plane 0.62 -> 0.84 ms, a list of 40,604 seeds 0.45 -> 0.56 ms). Whole lines, one after the other, are spread less
 //     below 16 lanes: 8,000 seeds of a list in a 64x64x64 cube 0.160 ms with 8
 //     lanes and 0.177 with 4, 128x128 seeds of its bottom 0.287 ms with 16, 0.295
 //     with 8 and 0.290 with 32. The FP64 tracer of Method I gives a line eight
@@ -665,7 +664,7 @@ Spread spread_of(const fqsl_field f, const fqsl_params *p, int bps, long long li
     if (f32 && may_split && kind == kSeedsList) r.split = 2 * lines <= warps;
     const long long items = (r.split ? 2 : 1) * lines;
     const int per = lanes_per_line(p);
-    const long long most = !f32 && per == 1 ? f->sms : (f32 && kind == kSeedsFace ? warps + warps / 16 : warps);
+    const long long most = !f32 && per == 1 ? f->sms : warps;
     // below 16 lanes, whole lines wait until they would fill half of the warps only
     const bool half = f32 && !r.split;
     if (p->chunk_tiles == 0 || per > 1)
