@@ -597,6 +597,7 @@ struct Spread {
     int bps;     // resident 128-thread blocks per SM
     int lanes;   // lanes of a warp that take lines
     bool split;  // the two directions of a line as separate items (FP32)
+    long long split_most;  // the most lines that a launch of this kind splits
 };
 
 // What kind of seeds a launch has.
@@ -656,12 +657,13 @@ Spread spread_of(const fqsl_field f, const fqsl_params *p, int bps, long long li
                  bool may_split)
 {
     const bool f32 = p->precision != FQSL_F64;
-    Spread r{bps, 32, false};
+    Spread r{bps, 32, false, 0};
     if (p->blocks_per_sm > 0) r.bps = p->blocks_per_sm < bps ? p->blocks_per_sm : bps;
     else if (f32 && lines > (long long)f->sms * kTraceBlock) r.bps = tlb_blocks((size_t)f->g.nodes * 32, kind, sparse, bps);
     const long long warps = (long long)f->sms * r.bps * (kTraceBlock / 32);
-    if (f32 && may_split && kind == kSeedsInside) r.split = lines <= (p->method == 2 ? 16 : 96) * warps;
-    if (f32 && may_split && kind == kSeedsList) r.split = 2 * lines <= warps;
+    if (f32 && may_split && kind == kSeedsInside) r.split_most = (p->method == 2 ? 16 : 96) * warps;
+    if (f32 && may_split && kind == kSeedsList) r.split_most = warps / 2;
+    r.split = lines <= r.split_most;
     const long long items = (r.split ? 2 : 1) * lines;
     const int per = lanes_per_line(p);
     const long long most = !f32 && per == 1 ? f->sms : warps;
@@ -772,6 +774,17 @@ Scratch layout(char *base, long long n, bool rot, bool lattice, bool f32, bool m
     }
     s.bytes = c.off;
     return s;
+}
+
+// Scratch of a call: what its layout takes, and never less than a smaller call
+// of the same kind that splits its directions would, so that calls up to the
+// largest one made so far find their scratch in place.
+size_t scratch_bytes(const Spread &sp, long long n, bool rot, bool lattice, bool f32, bool m2)
+{
+    const size_t own = layout(nullptr, n, rot, lattice, f32, m2, sp.split).bytes;
+    if (sp.split || sp.split_most < 1) return own;
+    const size_t split = layout(nullptr, n < sp.split_most ? n : sp.split_most, rot, lattice, f32, m2, true).bytes;
+    return own > split ? own : split;
 }
 
 fqsl_status ensure_scratch(fqsl_field f, size_t bytes)
@@ -1080,8 +1093,7 @@ fqsl_status run_qmap_locked(fqsl_field f, const Lattice &lat0, const fqsl_params
         tl = tape_layout_of(tape, (char *)tape->buf, tape->pool);
         s = tl.s;
     } else {
-        Scratch sz = layout(nullptr, n, rot, true, f32, m2, sp.split);
-        fqsl_status st = ensure_scratch(f, sz.bytes);
+        fqsl_status st = ensure_scratch(f, scratch_bytes(sp, n, rot, true, f32, m2));
         if (st != FQSL_OK) return st;
         s = layout((char *)f->scratch, n, rot, true, f32, m2, sp.split);
     }
@@ -1361,8 +1373,7 @@ fqsl_status fqsl_twist(fqsl_field f, const double *seeds_dev, long long n, const
     const bool f32 = p->precision != FQSL_F64;
     std::lock_guard<std::mutex> lock(f->mu);
     const Spread sp = spread_of(f, p, blocks_per_sm(f, p->precision, kSrcList, p->scheme), n, kSeedsList, true, true);
-    Scratch sz = layout(nullptr, n, false, false, f32, false, sp.split);
-    st = ensure_scratch(f, sz.bytes);
+    st = ensure_scratch(f, scratch_bytes(sp, n, false, false, f32, false));
     if (st != FQSL_OK) return st;
     Scratch s = layout((char *)f->scratch, n, false, false, f32, false, sp.split);
     cudaError_t e = cudaMemsetAsync(s.ctr, 0, s.zero_bytes, stream);
