@@ -1914,9 +1914,10 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A0, const BatchArgs 
         // leaves by: every line of a face plane has one) evaluates the same point
         // at every stage, so the first stage's values serve all of them: 128x128
         // seeds of a 64x64x64 cube 291 -> 282 us. (Not the 3/8 rule: 91,000 seeds
-        // 787 us with it, 772 at most without; nor the taped tracer, where its
+        // 787 us with it, 772 at most without; nor Method II, whose code outgrows the
+        // instruction cache already; nor the taped tracer, where its
         // registers cost the longest line 1 %.)
-        const bool still = SCH == 0 && !TAPE && henon && hh == (T)0;
+        const bool still = SCH == 0 && DEV == 0 && !TAPE && henon && hh == (T)0;
         T o[NS];
 #pragma unroll
         for (int s = 0; s < NST; s++) {
