@@ -89,6 +89,7 @@ struct fqsl_field_s {
     unsigned long long *counters = nullptr;  // [0] primary head, [1] extra head, [2] rotated count (low 32 bits),
                                              // [4] first failed index check of the adjoint kernels, [5] their count
     int blocks_cache[2][3][3] = {};  // [scheme][precision][source] resident blocks per SM
+    int blocks_cache_lane[2] = {};   // FP64 lattices with a lane per line: [scheme]
     int blocks_cache_m2[2][2][2] = {};  // Method II: [scheme][fp64][way - 1]
     int blocks_cache_tape[2][3][2] = {};  // taped tracers: [scheme][precision][lattice, extra]
     bool timing = false, timed = false, extra_timed = false;
@@ -595,6 +596,7 @@ DevParams dev_params(const fqsl_params *p)
 // How an untaped launch spreads its lines over the GPU.
 struct Spread {
     int bps;     // resident 128-thread blocks per SM
+    int per;     // lanes of a line
     int lanes;   // lanes of a warp that take lines
     bool split;  // the two directions of a line as separate items (FP32)
     long long split_most;  // the most lines that a launch of this kind splits
@@ -653,11 +655,37 @@ int tlb_blocks(size_t record_bytes, SeedKind kind, bool sparse, int bps)
 //     narrow FP64 pipe the same time whatever their lanes.
 int lanes_per_line(const fqsl_params *p) { return p->precision == FQSL_F64 && p->method == 1 ? 8 : 1; }
 
-Spread spread_of(const fqsl_field f, const fqsl_params *p, int bps, long long lines, SeedKind kind, bool sparse,
+// Does an FP64 plane of Method I give a line one lane (trace64_lane.cu) and not
+// eight? Eight are faster until the longest lines no longer matter, and on a
+// grid of spacing 1 with adaptive steps always (4 million seeds of a 256x256x128
+// cube: 304 against 322 ms): each stage's three quotients by the cell widths are
+// dearer on the integer pipe, and a fixed step has no error to form, no step to
+// choose and no rejected trials between its stages. Lines here in units of the
+// 1,024 lanes an SM can hold; measured (128x128x64 to 512x512x256 cubes) with
+// eight lanes against one, time ratio at 0.49 / 1.0 / 2.0 / 4.0 million seeds:
+//   other grids, adaptive   face 0.68-0.84 / 0.87-0.98 / 0.94-1.04 / 0.99-1.09
+//                           inside 0.87-0.91 / 1.02 / 1.06-1.10 / -
+//   other grids, fixed      face 0.74-0.84 / 1.04-1.09 / 1.10-1.15 / 1.13-1.19
+//                           inside 0.69-1.02 / - / 0.99-1.19 / -
+//   spacing 1, fixed        face 0.64-0.79 / 0.95-0.98 / 1.01-1.02 / 1.04-1.05
+//                           inside 0.67-0.79 / 1.00-1.01 / 0.94-1.03 / 1.05-1.06
+// With the rule 4 million seeds of the bottom of an anisotropic 256x256x128 cube
+// take 421 -> 355 ms (fixed step) and 327 -> 294 ms, of a stretched one 765 -> 679 ms
+// and 521 -> 486 ms. Volumes (lines of all lengths in each warp) keep eight: 0.69-0.80
+// at 8 million seeds; so do lists and, below 2 million lines, batches and taped maps.
+bool line_per_lane(const fqsl_field f, const fqsl_params *p, const Lattice &lat, bool face)
+{
+    if (p->precision != FQSL_F64 || p->method != 1 || lat.n3 > 1) return false;
+    const long long n = lat.n1 * lat.n2, full = (long long)f->sms * 1024;
+    if (f->g.unit) return p->scheme == 1 && n >= (face ? 8 : 16) * full;
+    return n >= (p->scheme == 0 && face ? 8 : 6) * full;
+}
+
+Spread spread_of(const fqsl_field f, const fqsl_params *p, int per, int bps, long long lines, SeedKind kind, bool sparse,
                  bool may_split)
 {
     const bool f32 = p->precision != FQSL_F64;
-    Spread r{bps, 32, false, 0};
+    Spread r{bps, per, 32, false, 0};
     if (p->blocks_per_sm > 0) r.bps = p->blocks_per_sm < bps ? p->blocks_per_sm : bps;
     else if (f32 && lines > (long long)f->sms * kTraceBlock) r.bps = tlb_blocks((size_t)f->g.nodes * 32, kind, sparse, bps);
     const long long warps = (long long)f->sms * r.bps * (kTraceBlock / 32);
@@ -665,7 +693,6 @@ Spread spread_of(const fqsl_field f, const fqsl_params *p, int bps, long long li
     if (f32 && may_split && kind == kSeedsList) r.split_most = warps / 2;
     r.split = lines <= r.split_most;
     const long long items = (r.split ? 2 : 1) * lines;
-    const int per = lanes_per_line(p);
     const long long most = !f32 && per == 1 ? f->sms : warps;
     // below 16 lanes, whole lines wait until they would fill half of the warps only
     const bool half = f32 && !r.split;
@@ -824,28 +851,37 @@ int blocks_per_sm(fqsl_field f, int precision, int src, int p_scheme)
     return c;
 }
 
+int lane_blocks_per_sm(fqsl_field f, int scheme)
+{
+    int &c = f->blocks_cache_lane[scheme];
+    if (!c) c = trace64_lane_blocks_per_sm(f->g.rect != 0, scheme);
+    return c;
+}
+
 // The grid of a launch of `items` items spread as sp says; full: lines that the
 // host cannot count follow (extra lines), so the grid fills the GPU.
-long long spread_grid(const fqsl_params *p, const Spread &sp, int sms, long long items, bool full)
+long long spread_grid(const Spread &sp, int sms, long long items, bool full)
 {
     long long grid = (long long)sms * sp.bps;
-    const long long per_block = (long long)(sp.lanes / lanes_per_line(p)) * (kTraceBlock / 32);
+    const long long per_block = (long long)(sp.lanes / sp.per) * (kTraceBlock / 32);
     const long long need = ((sp.split ? 2 : 1) * items + per_block - 1) / per_block;
     if (!full && need < grid) grid = need;
     return grid < 1 ? 1 : grid;
 }
 
-void set_spread(TraceArgs &a, const fqsl_params *p, const Spread &sp)
+void set_spread(TraceArgs &a, const Spread &sp)
 {
     a.p.lanes = sp.lanes;
     a.p.split = sp.split ? 1 : 0;
-    if (lanes_per_line(p) > 1) a.p.chunk = sp.lanes / lanes_per_line(p);
+    if (sp.per > 1) a.p.chunk = sp.lanes / sp.per;
     else if (sp.lanes < 32) a.p.chunk = sp.lanes;
     else if (sp.split) a.p.chunk = kTileU * kTileV;
 }
 
-cudaError_t launch_trace(const fqsl_params *p, const TraceArgs &a, int src, long long grid, cudaStream_t s)
+cudaError_t launch_trace(const fqsl_params *p, const TraceArgs &a, const Spread &sp, int src, long long grid,
+                         cudaStream_t s)
 {
+    if (sp.per < lanes_per_line(p)) return launch_trace64_lane(a, (int)grid, s);
     return p->precision == FQSL_F64 ? launch_trace_f64(a, src, (int)grid, kTraceBlock, s)
                                     : launch_trace_f32(a, src, (int)grid, kTraceBlock, s,
                                                        p->precision == FQSL_F32_ACC64);
@@ -853,16 +889,22 @@ cudaError_t launch_trace(const fqsl_params *p, const TraceArgs &a, int src, long
 
 // The extra lines of rotated seeds in a launch of their own: the FP32 lattice
 // kernel with no lattice items, the FP64 one's own source.
-cudaError_t launch_extra(fqsl_field f, const fqsl_params *p, TraceArgs a, const Scratch &s, const Spread &sp,
+cudaError_t launch_extra(fqsl_field f, const fqsl_params *p, TraceArgs a, const Scratch &s, Spread sp,
                          cudaStream_t stream)
 {
     a.q.head = s.ctr + 1;
     const bool f32 = p->precision != FQSL_F64;
+    if (sp.per < lanes_per_line(p)) {  // the lattice's lines had a lane each
+        sp.per = lanes_per_line(p);
+        sp.bps = blocks_per_sm(f, p->precision, kSrcExtra, p->scheme);
+        if (p->blocks_per_sm > 0 && p->blocks_per_sm < sp.bps) sp.bps = p->blocks_per_sm;
+        set_spread(a, sp);
+    }
     if (f32) {
         a.nitems = 0;
         a.p.merge = 1;
     }
-    return launch_trace(p, a, f32 ? kSrcLattice : kSrcExtra, spread_grid(p, sp, f->sms, 0, true), stream);
+    return launch_trace(p, a, sp, f32 ? kSrcLattice : kSrcExtra, spread_grid(sp, f->sms, 0, true), stream);
 }
 
 int blocks_per_sm_m2(fqsl_field f, const fqsl_params *p)
@@ -1068,9 +1110,13 @@ fqsl_status run_qmap_locked(fqsl_field f, const Lattice &lat0, const fqsl_params
     Scratch s;
     Spread sp{};
     TapeLayout tl{};
-    if (!tape)
-        sp = spread_of(f, p, m2 ? blocks_per_sm_m2(f, p) : blocks_per_sm(f, p->precision, kSrcLattice, p->scheme), n,
-                       face_plane ? kSeedsFace : kSeedsInside, sparse_lattice(f->g, lat), true);
+    if (!tape) {
+        const bool lane = line_per_lane(f, p, lat, face_plane);
+        const int bps = m2 ? blocks_per_sm_m2(f, p)
+                           : (lane ? lane_blocks_per_sm(f, p->scheme) : blocks_per_sm(f, p->precision, kSrcLattice, p->scheme));
+        sp = spread_of(f, p, lane ? 1 : lanes_per_line(p), bps, n, face_plane ? kSeedsFace : kSeedsInside,
+                       sparse_lattice(f->g, lat), true);
+    }
     if (tape) {
         tape->valid = false;
         tape->field = f;
@@ -1126,7 +1172,7 @@ fqsl_status run_qmap_locked(fqsl_field f, const Lattice &lat0, const fqsl_params
     a.prep = s.prep;
     a.tape = tl.tape;
     a.nitems = lat.n3 * lat.tiles_u * lat.tiles_v * (long long)(kTileU * kTileV);
-    if (!tape) set_spread(a, p, sp);
+    if (!tape) set_spread(a, sp);
     // (with timing on, the extra lines get a launch of their own to be timed)
     a.p.merge = !tape && f32 && rot && !f->timing;
     if (f32) {
@@ -1136,7 +1182,7 @@ fqsl_status run_qmap_locked(fqsl_field f, const Lattice &lat0, const fqsl_params
     }
     mark(f, 0, stream);
     if (m2) {
-        e = launch_trace_m2(p, a, spread_grid(p, sp, f->sms, a.nitems, false), stream);
+        e = launch_trace_m2(p, a, spread_grid(sp, f->sms, a.nitems, false), stream);
         if (e != cudaSuccess) return cuda_fail(e, who);
         mark(f, 1, stream);
         mark(f, 2, stream);
@@ -1169,7 +1215,7 @@ fqsl_status run_qmap_locked(fqsl_field f, const Lattice &lat0, const fqsl_params
         if (grid < 1) grid = 1;
         e = launch_tape(a, p, kSrcLattice, grid, stream);
     } else {
-        e = launch_trace(p, a, kSrcLattice, spread_grid(p, sp, f->sms, a.nitems, a.p.merge != 0), stream);
+        e = launch_trace(p, a, sp, kSrcLattice, spread_grid(sp, f->sms, a.nitems, a.p.merge != 0), stream);
     }
     if (e != cudaSuccess) return cuda_fail(e, who);
     mark(f, 1, stream);
@@ -1372,7 +1418,8 @@ fqsl_status fqsl_twist(fqsl_field f, const double *seeds_dev, long long n, const
     cudaStream_t stream = (cudaStream_t)cuda_stream;
     const bool f32 = p->precision != FQSL_F64;
     std::lock_guard<std::mutex> lock(f->mu);
-    const Spread sp = spread_of(f, p, blocks_per_sm(f, p->precision, kSrcList, p->scheme), n, kSeedsList, true, true);
+    const Spread sp = spread_of(f, p, lanes_per_line(p), blocks_per_sm(f, p->precision, kSrcList, p->scheme), n,
+                                kSeedsList, true, true);
     st = ensure_scratch(f, scratch_bytes(sp, n, false, false, f32, false));
     if (st != FQSL_OK) return st;
     Scratch s = layout((char *)f->scratch, n, false, false, f32, false, sp.split);
@@ -1386,9 +1433,9 @@ fqsl_status fqsl_twist(fqsl_field f, const double *seeds_dev, long long n, const
     a.nitems = n;
     a.rec = s.rec;
     a.q.head = s.ctr;
-    set_spread(a, p, sp);
+    set_spread(a, sp);
     mark(f, 0, stream);
-    e = launch_trace(p, a, kSrcList, spread_grid(p, sp, f->sms, (n + 31) / 32 * 32, false), stream);
+    e = launch_trace(p, a, sp, kSrcList, spread_grid(sp, f->sms, (n + 31) / 32 * 32, false), stream);
     if (e != cudaSuccess) return cuda_fail(e, who);
     mark(f, 1, stream);
     mark(f, 2, stream);
@@ -1510,10 +1557,10 @@ extern "C" fqsl_status fqsl_qmap_plane_static(fqsl_field f, const double origin[
     const SeedKind kind = face_plane ? kSeedsFace : kSeedsInside;
     const bool sparse = sparse_lattice(f->g, lat);
     const int bps = blocks_per_sm(f, p->precision, kSrcLattice, p->scheme);
-    Spread sp = spread_of(f, p, bps, n, kind, sparse, true);
+    Spread sp = spread_of(f, p, lanes_per_line(p), bps, n, kind, sparse, true);
     Scratch need = layout(nullptr, n, rot, true, f32, false, sp.split);
     if (need.bytes > kStaticScratchBytes && sp.split) {
-        sp = spread_of(f, p, bps, n, kind, sparse, false);
+        sp = spread_of(f, p, lanes_per_line(p), bps, n, kind, sparse, false);
         need = layout(nullptr, n, rot, true, f32);
     }
     if (need.bytes > kStaticScratchBytes)
@@ -1537,7 +1584,7 @@ extern "C" fqsl_status fqsl_qmap_plane_static(fqsl_field f, const double origin[
     a.q.rot_slot = s.rot_slot;
     a.prep = s.prep;
     a.nitems = lat.n3 * lat.tiles_u * lat.tiles_v * (long long)(kTileU * kTileV);
-    set_spread(a, p, sp);
+    set_spread(a, sp);
     a.p.merge = f32 && rot && !f->timing;
     if (f32) {
         e = launch_seed_prep_f32(a, n, stream);
@@ -1545,7 +1592,7 @@ extern "C" fqsl_status fqsl_qmap_plane_static(fqsl_field f, const double origin[
         if (e != cudaSuccess) return cuda_fail(e, who);
     }
     mark(f, 0, stream);
-    e = launch_trace(p, a, kSrcLattice, spread_grid(p, sp, f->sms, a.nitems, a.p.merge != 0), stream);
+    e = launch_trace(p, a, sp, kSrcLattice, spread_grid(sp, f->sms, a.nitems, a.p.merge != 0), stream);
     if (e != cudaSuccess) return cuda_fail(e, who);
     mark(f, 1, stream);
     if (rot && !a.p.merge) {

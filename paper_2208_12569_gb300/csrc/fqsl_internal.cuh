@@ -264,6 +264,9 @@ cudaError_t launch_loss(long long n, const double *Q, const double *Tw, const do
 cudaError_t launch_curl_pack(const void *B, fqsl_dtype bt, const FieldView &g, void *rec32, void *rec64,
                              cudaStream_t s);
 cudaError_t launch_trace_f32(const TraceArgs &a, int src, int grid, int block, cudaStream_t s, bool acc64);
+// a lattice with a lane per line (trace64_lane.cu); the other FP64 launches give a line eight
+cudaError_t launch_trace64_lane(const TraceArgs &a, int grid, cudaStream_t s);
+int trace64_lane_blocks_per_sm(bool rect, int scheme);
 cudaError_t launch_trace_f64(const TraceArgs &a, int src, int grid, int block, cudaStream_t s);
 // tracers that also write the step tape (a.tape; lattice or extra lines)
 cudaError_t launch_trace_tape_f32(const TraceArgs &a, int src, int grid, cudaStream_t s, bool acc64);
