@@ -609,8 +609,8 @@ enum SeedKind {
     kSeedsList     // an explicit list: neighbours in it need not be neighbours in space
 };
 
-// Blocks per SM. FP32 lines that share no cells (lists; lattices at least a
-// cell apart) touch pages of the node records all over a large cube, and more
+// Blocks per SM. FP32 lines that share no cells (lists; lattices two cells
+// apart) touch pages of the node records all over a large cube, and more
 // resident lanes than the address translation can serve make each load slower
 // than they hide: nothing but the latency is busy (ncu, 2.1 GB of records, 4
 // blocks: L1 24 %, L2 19 %, DRAM 25 %; 2 blocks are 1.4 times as fast with the
@@ -621,7 +621,14 @@ enum SeedKind {
 //   0.91 GB   7.76 /  7.44 /  9.02          7.41 /  6.48 /  5.71
 //   1.44 GB  14.22 /  9.20 / 10.70          9.96 /  8.67 /  7.17
 //   2.15 GB  20.01 / 11.83 / 12.49         12.19 / 10.58 /  8.53
-// (a plane of 1024x512 seeds half a cell apart in the last cube: 5.43 / 5.86 / 7.40)
+// (a plane of 1024x512 seeds half a cell apart in the last cube: 5.43 / 5.86 / 7.40).
+// Lattices a given number of cells apart, at 4 / 3 blocks (1.34 GB; 2.0 GB):
+//   cells  plane inside               volume
+//   0.9    2.15 / 2.53; 2.67 / 3.09   0.87 / 0.95; 3.11 / 3.27
+//   1      2.24 / 2.56; 2.68 / 3.12   1.02 / 1.10; 3.45 / 3.58
+//   1.4    2.10 / 2.30; 2.98 / 3.15   1.86 / 1.91; 4.17 / 4.20
+//   2      2.11 / 1.80; 2.61 / 2.68   3.56 / 3.36; 4.19 / 3.80
+//   4      1.25 / 1.17; 2.01 / 1.71   6.24 / 4.17; 5.37 / 3.85
 int tlb_blocks(size_t record_bytes, SeedKind kind, bool sparse, int bps)
 {
     if (!sparse) return bps;
@@ -711,8 +718,8 @@ int tape_lanes(const fqsl_params *p, long long warps, long long items)
     return lanes;
 }
 
-// Are a lattice's seeds a cell or more apart (its 8x4-seed tile covers at
-// least as many cells as it has seeds)?
+// Are a lattice's seeds two cells or more apart (its 8x4-seed tile covers at
+// least four times as many cells as it has seeds)?
 bool sparse_lattice(const FieldView &g, const Lattice &lat)
 {
     double area = 1.0;
@@ -726,7 +733,7 @@ bool sparse_lattice(const FieldView &g, const Lattice &lat)
         }
         area *= s;
     }
-    return area >= 1.0;
+    return area >= 4.0;
 }
 
 struct Scratch {
