@@ -598,6 +598,7 @@ struct Spread {
     int bps;     // resident 128-thread blocks per SM
     int per;     // lanes of a line
     int lanes;   // lanes of a warp that take lines
+    int few;     // seed lists: blocks per SM if the seeds turn out scattered (0: bps in any case)
     bool split;  // the two directions of a line as separate items (FP32)
     long long split_most;  // the most lines that a launch of this kind splits
 };
@@ -606,7 +607,7 @@ struct Spread {
 enum SeedKind {
     kSeedsFace,    // a lattice on a face of the box: one direction of each line ends at once
     kSeedsInside,  // a lattice inside the box
-    kSeedsList     // an explicit list: neighbours in it need not be neighbours in space
+    kSeedsList     // an explicit list: whether neighbours in it are neighbours in space is seen on the device
 };
 
 // Blocks per SM. FP32 lines that share no cells (lists; lattices two cells
@@ -629,6 +630,15 @@ enum SeedKind {
 //   1.4    2.10 / 2.30; 2.98 / 3.15   1.86 / 1.91; 4.17 / 4.20
 //   2      2.11 / 1.80; 2.61 / 2.68   3.56 / 3.36; 4.19 / 3.80
 //   4      1.25 / 1.17; 2.01 / 1.71   6.24 / 4.17; 5.37 / 3.85
+// A list may hold a plane's or a curve's seeds in order. list_blocks (trace_f32.cu)
+// looks at pairs of neighbours spread over the list and holds it to the fewer
+// blocks only if most are more than 1.5 cells apart. Rows of 300,000 seeds, ms at 4 /
+// 3 / 2 blocks (the last column with 2 cells shuffled):
+//   records   0.5 cells apart      1 cell               2 cells              shuffled
+//   0.48 GB   1.19 / 1.31 / 1.64   1.05 / 1.14 / 1.43   1.61 / 1.55 / 1.92   2.96 / 2.60 / 2.90
+//   0.85 GB   1.69 / 1.82 / 2.25   1.81 / 1.64 / 2.01   3.26 / 2.44 / 2.62   4.88 / 4.12 / 4.05
+//   1.34 GB   1.44 / 1.59 / 1.99   1.71 / 1.65 / 2.08   3.38 / 2.35 / 2.37   5.32 / 4.48 / 4.21
+//   2.00 GB   1.32 / 1.47 / 1.85   1.80 / 1.97 / 2.46   2.90 / 2.02 / 2.26   5.57 / 4.67 / 4.49
 int tlb_blocks(size_t record_bytes, SeedKind kind, bool sparse, int bps)
 {
     if (!sparse) return bps;
@@ -692,10 +702,13 @@ Spread spread_of(const fqsl_field f, const fqsl_params *p, int per, int bps, lon
                  bool may_split)
 {
     const bool f32 = p->precision != FQSL_F64;
-    Spread r{bps, per, 32, false, 0};
-    if (p->blocks_per_sm > 0) r.bps = p->blocks_per_sm < bps ? p->blocks_per_sm : bps;
-    else if (f32 && lines > (long long)f->sms * kTraceBlock) r.bps = tlb_blocks((size_t)f->g.nodes * 32, kind, sparse, bps);
-    const long long warps = (long long)f->sms * r.bps * (kTraceBlock / 32);
+    Spread r{bps, per, 32, 0, false, 0};
+    int blocks = bps;  // blocks whose lanes the lines are spread over
+    if (p->blocks_per_sm > 0) blocks = p->blocks_per_sm < bps ? p->blocks_per_sm : bps;
+    else if (f32 && lines > (long long)f->sms * kTraceBlock) blocks = tlb_blocks((size_t)f->g.nodes * 32, kind, sparse, bps);
+    if (kind == kSeedsList && p->blocks_per_sm <= 0 && blocks < bps) r.few = blocks;
+    else r.bps = blocks;
+    const long long warps = (long long)f->sms * blocks * (kTraceBlock / 32);
     if (f32 && may_split && kind == kSeedsInside) r.split_most = (p->method == 2 ? 16 : 96) * warps;
     if (f32 && may_split && kind == kSeedsList) r.split_most = warps / 2;
     r.split = lines <= r.split_most;
@@ -737,7 +750,7 @@ bool sparse_lattice(const FieldView &g, const Lattice &lat)
 }
 
 struct Scratch {
-    unsigned long long *ctr = nullptr;  // [0], [1] work counters, [2] rotated seeds (low 32 bits)
+    unsigned long long *ctr = nullptr;  // [0], [1] work counters, [2] rotated seeds, [3] blocks of a list (low 32 bits)
     size_t zero_bytes = 0;              // from ctr on: cleared before the launch (counters, pair, rot_slot)
     LineRecs rec{}, ext{};
     SeedPrep prep{};
@@ -1442,6 +1455,11 @@ fqsl_status fqsl_twist(fqsl_field f, const double *seeds_dev, long long n, const
     a.q.head = s.ctr;
     set_spread(a, sp);
     mark(f, 0, stream);
+    if (sp.few) {
+        a.q.blocks = (unsigned int *)(s.ctr + 3);
+        e = launch_list_blocks(a, (unsigned)(f->sms * sp.few), stream);
+        if (e != cudaSuccess) return cuda_fail(e, who);
+    }
     e = launch_trace(p, a, sp, kSrcList, spread_grid(sp, f->sms, (n + 31) / 32 * 32, false), stream);
     if (e != cudaSuccess) return cuda_fail(e, who);
     mark(f, 1, stream);

@@ -133,6 +133,7 @@ struct Queue {
     unsigned int *rot_count;   // number of rotated seeds
     int32_t *rot_seed;         // rotated slot -> lattice index
     int32_t *rot_slot;         // lattice index -> slot + 1 (0 = not rotated)
+    unsigned int *blocks;      // seed lists: blocks of the launch that take lines (NULL: all)
 };
 
 enum Source { kSrcLattice = 0, kSrcExtra = 1, kSrcList = 2 };
@@ -330,6 +331,8 @@ constexpr int kTraceBlock = 128;
 cudaError_t launch_assemble(const AssembleArgs &a, cudaStream_t s);
 cudaError_t launch_assemble_f32(const AssembleArgs &a, cudaStream_t s);
 cudaError_t launch_seed_prep_f32(const TraceArgs &a, long long n, cudaStream_t s);
+// a.q.blocks: few if neighbours in the list a.seeds (a.nitems) lie scattered, else all
+cudaError_t launch_list_blocks(const TraceArgs &a, unsigned few, cudaStream_t s);
 // the extra lines of the rotated seeds that the pre-pass queued (DevParams::merge)
 cudaError_t launch_extra_prep_f32(const TraceArgs &a, cudaStream_t s);
 cudaError_t launch_extra_prep_rect_f32(const TraceArgs &a, unsigned grid, cudaStream_t s);

@@ -1744,6 +1744,9 @@ template <typename T, int SRC, bool ACC, int DEV = 0, bool BATCH = false, bool T
           int SCH = 0, bool FLEX = false>
 __device__ __forceinline__ void trace_body(const TraceArgs &A0, const BatchArgs &BA)
 {
+    if constexpr (SRC == kSrcList) {
+        if (A0.q.blocks && blockIdx.x >= *A0.q.blocks) return;
+    }
     constexpr bool SPLIT = TAPE && SRC == kSrcLattice;
     constexpr unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;

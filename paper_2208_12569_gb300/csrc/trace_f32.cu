@@ -67,6 +67,34 @@ int trace_blocks_per_sm_f32(int src, bool acc64) { return acc64 ? blocks<true>(s
 
 namespace fqsl {
 namespace {
+// Do the seeds of a list lie in order? 512 pairs of neighbours, spread evenly over
+// it, are asked whether they are within 1.5 cells (reach) of each other on every
+// axis. One block and one pair a thread: the loads' latency and the narrow FP64
+// pipe are what it takes (4,096 pairs added 25 us to a list of 1 ms).
+__global__ void __launch_bounds__(512) k_list_blocks(const double *__restrict__ seeds, long long n, double3 reach,
+                                                     unsigned few, unsigned *__restrict__ blocks)
+{
+    const double *p = seeds + 3 * ((n - 1) * (int)threadIdx.x / 512);
+    const bool near = fabs(p[3] - p[0]) <= reach.x && fabs(p[4] - p[1]) <= reach.y && fabs(p[5] - p[2]) <= reach.z;
+    const int count = __syncthreads_count(near);
+    if (threadIdx.x == 0) *blocks = 2 * count < 512 ? few : 0xffffffffu;
+}
+}  // namespace
+
+cudaError_t launch_list_blocks(const TraceArgs &a, unsigned few, cudaStream_t s)
+{
+    if (a.nitems < 2) return cudaErrorInvalidValue;
+    const FieldView &f = a.f;
+    const int n[3] = {f.nx, f.ny, f.nz};
+    double r[3];  // stretched grid: cells of the mean width
+    for (int c = 0; c < 3; c++) r[c] = 1.5 * (f.rect ? (f.hi64[c] - f.lo64[c]) / (n[c] - 1) : f.d[c]);
+    k_list_blocks<<<1, 512, 0, s>>>(a.seeds, a.nitems, make_double3(r[0], r[1], r[2]), few, a.q.blocks);
+    return cudaGetLastError();
+}
+}  // namespace fqsl
+
+namespace fqsl {
+namespace {
 __global__ void __launch_bounds__(256) k_seed_prep_f32(const TraceArgs A, long long n)
 {
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < n;

@@ -61,3 +61,34 @@ def test_lattice(field, apart, shape):
             fq.qmap_volume(f, (0.2, 0.2, 0.2), (apart,) * 3, w, h, d, p=p, out=out)
     limited, free = _ms(_calls(fq, call))
     assert limited < 1.0625 * free, (limited, free)
+
+
+def _rows(apart):
+    w, h = min(600, int((N[0] - 2) / apart)), min(500, int((N[1] - 2) / apart))
+    j, i = torch.meshgrid(torch.arange(h), torch.arange(w), indexing="ij")
+    return torch.stack((apart * i + 0.3, apart * j + 0.4, torch.full_like(i, 21.8, dtype=torch.float64)), -1).double().reshape(-1, 3)
+
+
+def _curves(g):
+    d = torch.randn((300, 1, 3), generator=g, dtype=torch.float64)
+    s = 0.3 * d / d.norm(dim=-1, keepdim=True) * torch.arange(1000.0).view(1, -1, 1)
+    s = s + torch.rand((300, 1, 3), generator=g, dtype=torch.float64) * torch.tensor(N, dtype=torch.float64)
+    return s.reshape(-1, 3).remainder(torch.tensor(N, dtype=torch.float64) - 1.0)
+
+
+@pytest.mark.parametrize("order", ["rows 0.5", "rows 1", "curves", "rows 3", "rows 1 shuffled"])
+def test_list(field, order):
+    fq, f = field
+    g = torch.Generator().manual_seed(1)
+    seeds = _curves(g) if order == "curves" else _rows(float(order.split()[1]))
+    if "shuffled" in order:
+        seeds = seeds[torch.randperm(seeds.shape[0], generator=g)]
+    seeds = seeds.cuda()
+    out = [fq.alloc_out(seeds.shape[0], q=False) for _ in range(2)]
+    fns = [lambda p=fq.params(precision="f32", blocks_per_sm=b), o=o: fq.twist(f, seeds, p, o) for b, o in zip((0, 8), out)]
+    limited, free = _ms(fns)
+    # rows 3 cells apart and scattered seeds run with fewer blocks, which has to pay
+    assert limited < (0.95 if order in ("rows 3", "rows 1 shuffled") else 1.0625) * free, (limited, free)
+    for k, t in out[0].items():
+        if t is not None:
+            assert t.cpu().numpy().tobytes() == out[1][k].cpu().numpy().tobytes(), k
