@@ -1287,7 +1287,8 @@ __device__ __forceinline__ void start_second(const TraceArgs &A, Lane<T> &L)
 // record as one lane tracing both directions would have: a bad first direction
 // ends the line (end 2 is the seed, only the first direction's trials count),
 // and if both together reach max_steps the second direction is traced again
-// with what the first left of the budget. Returns whether this lane has to.
+// with what the first left of the budget (a second direction that outlives the
+// first has joined it before, see split_adopt). Returns whether this lane has to.
 template <typename T, bool ACC, int DEV>
 __device__ __forceinline__ bool split_join(const TraceArgs &A, const LineRecs &R, Lane<T> &L, bool bad)
 {
@@ -1316,6 +1317,41 @@ __device__ __forceinline__ bool split_join(const TraceArgs &A, const LineRecs &R
     R.st[L.line] = (uint8_t)(st0 | st1);
     R.steps[L.line] = (int32_t)(both & 0xffffffffull);
     return false;
+}
+
+// The second direction of a split line, 128 trials after it last asked: is the
+// first one done? Then this lane takes the line over as one that traced both
+// directions, the first one's trials and status included, so that a line that
+// runs into max_steps does so with its whole budget known. (Left to split_join such
+// a line was traced twice: a volume of 64x64x32 seeds of a 512x512x128 cube whose
+// longest line is trapped, 425 ms; with this 209.)
+__device__ __forceinline__ bool split_first_done(const LineRecs &R, long long line)
+{
+    return (*(volatile unsigned long long *)(R.pair + line) >> 48) & 1ull;
+}
+
+// Returns whether the lane goes on (its position may be the seed again).
+template <typename T, bool ACC, int DEV>
+__device__ __forceinline__ bool split_adopt(const TraceArgs &A, const LineRecs &R, Lane<T> &L)
+{
+    __threadfence();
+    const unsigned long long w = *(volatile unsigned long long *)(R.pair + L.line);
+    const int st0 = (int)(w >> 32) & 0xff;
+    const int32_t steps0 = *(volatile int32_t *)(R.steps + L.line);
+    if ((w >> 50) & 1ull) {
+        write_end32(R, L.line, 1, (float)L.sx, (float)L.sy, (float)L.sz, -1);
+        R.st[L.line] = (uint8_t)st0;
+        return false;
+    }
+    if ((long long)steps0 + L.steps > A.p.max_steps) {
+        L.st = st0 | (L.st & kLaneExtra);
+        L.steps = steps0;
+        start_second<T, ACC, DEV>(A, L);
+        return true;
+    }
+    L.st = (L.st & ~kLaneSplit) | st0;
+    L.steps += steps0;
+    return true;
 }
 
 // Finish the line with a bad status (MAXSTEPS or NULL_B): the unfinished end
@@ -1895,6 +1931,12 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A0, const BatchArgs 
         const T sgn = (L.end == 0) ? -L.s0 : L.s0;
         T hh;
         if (!henon) {
+            if constexpr (FLEX) {
+                if ((L.steps & 127) == 127 && (L.st & kLaneSplit) && L.end == 1 && split_first_done(R, L.line)) {
+                    active = split_adopt<T, ACC, DEV>(A, R, L);
+                    continue;
+                }
+            }
             if (L.steps >= max_steps) {
                 active = finish_bad<T, ACC, DEV, SPLIT, RECT, FLEX>(A, R, L, FQSL_LINE_MAXSTEPS);
                 continue;
