@@ -1805,8 +1805,13 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A0, const BatchArgs 
     const bool psplit = FLEX && A0.p.split;
     if (psplit) nitems = 2 * ((nitems + 31) & ~31LL);
     // lanes of the warp that take lines (fewer than 32 where the lines would
-    // not fill the GPU's warps; see api.cu)
-    const unsigned gmask = A0.p.lanes >= 32 ? FULL : (1u << A0.p.lanes) - 1u;
+    // not fill the GPU's warps; see api.cu). The host could not count the extra
+    // lines: with them the lines may fill more lanes (48x48 seeds, all rotated:
+    // 0.52 ms with the lattice's two lanes, 0.22 with sixteen).
+    int take = A0.p.lanes;
+    if (MERGED && A0.p.merge)
+        while (take < 32 && nitems > (long long)gridDim.x * (blockDim.x / 32) * take) take *= 2;
+    const unsigned gmask = take >= 32 ? FULL : (1u << take) - 1u;
 
     long long ck_cur = 0, ck_end = 0, ck_base = 0;
     int ck_ent = 0;
@@ -1830,7 +1835,8 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A0, const BatchArgs 
         while (refill && idle != 0u && !exhausted) {
             if (ck_cur >= ck_end) {
                 unsigned long long base = 0;
-                const long long chunk = A0.p.chunk;  // (at most 32 with BATCH or p.split)
+                // (at most 32 with BATCH or p.split)
+                const long long chunk = MERGED && A0.p.lanes < 32 ? __popc(gmask) : A0.p.chunk;
                 if (lane == 0) base = atomicAdd(A0.q.head, (unsigned long long)chunk);
                 base = __shfl_sync(FULL, base, 0);
                 if ((long long)base >= nitems) {

@@ -575,11 +575,16 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A0, const BatchArgs 
     const Place g{0xffu << lead, lane & (kGroup - 1), lane & 3};
     const double hmin = A0.p.hmin, hmax = A0.p.hmax, graze = A0.p.graze;
     const int max_steps = (int)A0.p.max_steps;
-    const unsigned gmask = 0x01010101u & (A0.p.lanes >= 32 ? kFull : (1u << A0.p.lanes) - 1u);
 
     long long nitems = A0.nitems;
     if (BATCH) nitems = BA.ibase[BA.nent];
     else if (SRC == kSrcExtra) nitems = 4LL * (long long)(*(volatile unsigned *)A0.q.rot_count);
+    // lanes that take lines: the host chose them by the lattice's lines, and there
+    // may be four times as many extra lines (48x48 seeds, all rotated: 5.9 -> 4.0 ms)
+    int take = A0.p.lanes, chunk = A0.p.chunk;  // (chunk divides 32 with BATCH)
+    if (SRC == kSrcExtra)
+        for (; take < 32 && nitems > (long long)gridDim.x * (blockDim.x / 32) * chunk; chunk *= 2) take *= 2;
+    const unsigned gmask = 0x01010101u & (take >= 32 ? kFull : (1u << take) - 1u);
 
     long long ck_cur = 0, ck_end = 0, ck_base = 0;
     int ck_ent = 0, eb = 0;
@@ -597,7 +602,6 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A0, const BatchArgs 
         while (idle != 0u && !exhausted) {
             if (ck_cur >= ck_end) {
                 unsigned long long base = 0;
-                const long long chunk = A0.p.chunk;  // (divides 32 with BATCH)
                 if (lane == 0) base = atomicAdd(A0.q.head, (unsigned long long)chunk);
                 base = __shfl_sync(kFull, base, 0);
                 if ((long long)base >= nitems) {
