@@ -178,29 +178,29 @@ __device__ __forceinline__ Unit bhat(const TI *__restrict__ B, long long q)
 
 // grad(B/|B|) at the nodes for Method II way 1 (Sec. 4, Eq. grad_B): G[a*3+b]
 // = d(B_b/|B|)/dx_a with the stencils of the curl grid (RECT: node_diff_rect's).
-// A block holds B/|B| of a tile of 16 x 8 x 4 nodes and its one-node halo in
+// A block holds B/|B| of a tile of GX x GY x GZ nodes and its one-node halo in
 // shared memory, so that a node's is formed about twice and not 18 times (its
 // root and divisions are what the kernel spends its time on: repacking 256x256x128
 // nodes with the gradient took 9.54 ms when a thread formed all of a node's
 // differences from B, and takes 1.54 ms); the one-sided differences on the
 // faces, which reach two nodes, form theirs.
-constexpr int kGx = 16, kGy = 8, kGz = 4;
+constexpr int kGradThreads = 128;
 
-template <typename TI, bool RECT>
-__global__ void __launch_bounds__(kGx *kGy) k_gradb_pack(const TI *__restrict__ B, const FieldView g,
-                                                         float4 *__restrict__ g32, double *__restrict__ g64)
+template <typename TI, bool RECT, int GX, int GY, int GZ>
+__global__ void __launch_bounds__(kGradThreads) k_gradb_pack(const TI *__restrict__ B, const FieldView g,
+                                                             float4 *__restrict__ g32, double *__restrict__ g64)
 {
-    __shared__ double U[3][kGz + 2][kGy + 2][kGx + 2];
+    __shared__ double U[3][GZ + 2][GY + 2][GX + 2];
     const int nx = g.nx, ny = g.ny, nz = g.nz;
     const long long stride[3] = {1, nx, (long long)nx * ny};
     const int n[3] = {nx, ny, nz};
-    const int tx = (nx + kGx - 1) / kGx, ty = (ny + kGy - 1) / kGy;
-    const long long tiles = (long long)tx * ty * ((nz + kGz - 1) / kGz);
+    const int tx = (nx + GX - 1) / GX, ty = (ny + GY - 1) / GY;
+    const long long tiles = (long long)tx * ty * ((nz + GZ - 1) / GZ);
     for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
-        const int x0 = (int)(t % tx) * kGx, y0 = (int)(t / tx % ty) * kGy, z0 = (int)(t / ((long long)tx * ty)) * kGz;
+        const int x0 = (int)(t % tx) * GX, y0 = (int)(t / tx % ty) * GY, z0 = (int)(t / ((long long)tx * ty)) * GZ;
         __syncthreads();
-        for (int q = threadIdx.x; q < (kGz + 2) * (kGy + 2) * (kGx + 2); q += kGx * kGy) {
-            const int i = q % (kGx + 2), j = q / (kGx + 2) % (kGy + 2), k = q / ((kGx + 2) * (kGy + 2));
+        for (int q = threadIdx.x; q < (GZ + 2) * (GY + 2) * (GX + 2); q += kGradThreads) {
+            const int i = q % (GX + 2), j = q / (GX + 2) % (GY + 2), k = q / ((GX + 2) * (GY + 2));
             const int x = x0 + i - 1, y = y0 + j - 1, z = z0 + k - 1;
             if (x < 0 || y < 0 || z < 0 || x >= nx || y >= ny || z >= nz) continue;
             const Unit u = bhat(B, x + nx * (y + (long long)ny * z));
@@ -208,10 +208,10 @@ __global__ void __launch_bounds__(kGx *kGy) k_gradb_pack(const TI *__restrict__ 
             for (int c = 0; c < 3; c++) U[c][k][j][i] = u.v[c];
         }
         __syncthreads();
-        const int i = threadIdx.x % kGx, j = threadIdx.x / kGx;
-        if (x0 + i >= nx || y0 + j >= ny) continue;
 #pragma unroll 1
-        for (int k = 0; k < kGz && z0 + k < nz; k++) {
+        for (int q = threadIdx.x; q < GX * GY * GZ; q += kGradThreads) {
+            const int i = q % GX, j = q / GX % GY, k = q / (GX * GY);
+            if (x0 + i >= nx || y0 + j >= ny || z0 + k >= nz) continue;
             const int at[3] = {x0 + i, y0 + j, z0 + k};
             const long long node = at[0] + nx * (at[1] + (long long)ny * at[2]);
             double G[3][3];
@@ -278,6 +278,22 @@ __global__ void __launch_bounds__(kGx *kGy) k_gradb_pack(const TI *__restrict__ 
     }
 }
 
+template <typename TI, bool RECT, int GX, int GY, int GZ>
+void gradb_tiled(const void *B, const FieldView &g, float4 *g32, double *g64, int sms, cudaStream_t s)
+{
+    const long long tiles = (long long)((g.nx + GX - 1) / GX) * ((g.ny + GY - 1) / GY) * ((g.nz + GZ - 1) / GZ);
+    const unsigned blocks = (unsigned)(tiles < (long long)sms * 32 ? tiles : (long long)sms * 32);
+    k_gradb_pack<TI, RECT, GX, GY, GZ><<<blocks, kGradThreads, 0, s>>>((const TI *)B, g, g32, g64);
+}
+
+template <typename TI, bool RECT>
+void gradb_tiles(int shape, const void *B, const FieldView &g, float4 *g32, double *g64, int sms, cudaStream_t s)
+{
+    if (shape == 0) gradb_tiled<TI, RECT, 16, 8, 4>(B, g, g32, g64, sms, s);
+    else if (shape == 1) gradb_tiled<TI, RECT, 4, 32, 4>(B, g, g32, g64, sms, s);
+    else gradb_tiled<TI, RECT, 4, 4, 32>(B, g, g32, g64, sms, s);
+}
+
 }  // namespace
 
 cudaError_t launch_gradb_pack(const void *B, fqsl_dtype bt, const FieldView &g, void *grad32, void *grad64,
@@ -286,14 +302,15 @@ cudaError_t launch_gradb_pack(const void *B, fqsl_dtype bt, const FieldView &g, 
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const long long tiles = (long long)((g.nx + kGx - 1) / kGx) * ((g.ny + kGy - 1) / kGy) * ((g.nz + kGz - 1) / kGz);
-    const unsigned blocks = (unsigned)(tiles < (long long)sms * 32 ? tiles : (long long)sms * 32);
-    float4 *o32 = (float4 *)grad32;
-    double *o64 = (double *)grad64;
-    if (bt == FQSL_F32 && g.rect) k_gradb_pack<float, true><<<blocks, kGx * kGy, 0, s>>>((const float *)B, g, o32, o64);
-    else if (bt == FQSL_F32) k_gradb_pack<float, false><<<blocks, kGx * kGy, 0, s>>>((const float *)B, g, o32, o64);
-    else if (g.rect) k_gradb_pack<double, true><<<blocks, kGx * kGy, 0, s>>>((const double *)B, g, o32, o64);
-    else k_gradb_pack<double, false><<<blocks, kGx * kGy, 0, s>>>((const double *)B, g, o32, o64);
+    // Tiles of 16 x 8 x 4 nodes; where an axis would leave most of that empty, of
+    // 4 x 32 x 4 or 4 x 4 x 32 (four updates of an FP32 cube of 2 x 512 x 512 nodes with
+    // the gradient 3.3 -> 1.03 ms, of 2 x 2 x 40,000 2.5 -> 0.77).
+    const int shape = g.nx > 8 ? 0 : (g.ny > 8 ? 1 : 2);
+    const bool f32 = bt == FQSL_F32;
+    if (f32 && g.rect) gradb_tiles<float, true>(shape, B, g, (float4 *)grad32, (double *)grad64, sms, s);
+    else if (f32) gradb_tiles<float, false>(shape, B, g, (float4 *)grad32, (double *)grad64, sms, s);
+    else if (g.rect) gradb_tiles<double, true>(shape, B, g, (float4 *)grad32, (double *)grad64, sms, s);
+    else gradb_tiles<double, false>(shape, B, g, (float4 *)grad32, (double *)grad64, sms, s);
     return cudaGetLastError();
 }
 
