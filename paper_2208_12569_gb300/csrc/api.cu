@@ -600,7 +600,7 @@ struct Spread {
     int lanes;   // lanes of a warp that take lines
     int few;     // seed lists: blocks per SM if the seeds turn out scattered (0: bps in any case)
     bool split;  // the two directions of a line as separate items (FP32)
-    long long split_most;  // the most lines that a launch of this kind splits
+    long long split_most;  // the most lines that any launch of this kind splits
 };
 
 // What kind of seeds a launch has.
@@ -709,9 +709,11 @@ Spread spread_of(const fqsl_field f, const fqsl_params *p, int per, int bps, lon
     if (kind == kSeedsList && p->blocks_per_sm <= 0 && blocks < bps) r.few = blocks;
     else r.bps = blocks;
     const long long warps = (long long)f->sms * blocks * (kTraceBlock / 32);
-    if (f32 && may_split && kind == kSeedsInside) r.split_most = (p->method == 2 ? 16 : 96) * warps;
-    if (f32 && may_split && kind == kSeedsList) r.split_most = warps / 2;
-    r.split = lines <= r.split_most;
+    const long long most_of_warps = kind == kSeedsList ? 0 : (p->method == 2 ? 16 : 96);
+    const long long all_warps = (long long)f->sms * bps * (kTraceBlock / 32);
+    if (f32) r.split_most = kind == kSeedsList ? all_warps / 2 : most_of_warps * all_warps;
+    r.split = f32 && may_split && kind != kSeedsFace &&
+              lines <= (kind == kSeedsList ? warps / 2 : most_of_warps * warps);
     const long long items = (r.split ? 2 : 1) * lines;
     const long long most = !f32 && per == 1 ? f->sms : warps;
     // below 16 lanes, whole lines wait until they would fill half of the warps only
@@ -823,9 +825,10 @@ Scratch layout(char *base, long long n, bool rot, bool lattice, bool f32, bool m
     return s;
 }
 
-// Scratch of a call: what its layout takes, and never less than a smaller call
-// of the same kind that splits its directions would, so that calls up to the
-// largest one made so far find their scratch in place.
+// Scratch of a call: what its layout takes, and never less than any smaller call
+// of the same kind that splits its directions would, whatever its seeds' place and
+// spacing and its blocks_per_sm, so that calls up to the largest one made so far
+// find their scratch in place.
 size_t scratch_bytes(const Spread &sp, long long n, bool rot, bool lattice, bool f32, bool m2)
 {
     const size_t own = layout(nullptr, n, rot, lattice, f32, m2, sp.split).bytes;
@@ -848,6 +851,53 @@ fqsl_status ensure_scratch(fqsl_field f, size_t bytes)
         return cuda_fail(e, "scratch allocation");
     }
     f->scratch_cap = bytes;
+    return FQSL_OK;
+}
+
+// Is anything captured that an allocation would break?
+bool capturing(cudaStream_t stream)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &cs) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return cs != cudaStreamCaptureStatusNone;
+}
+
+// Scratch of an untaped call and its layout. whole: the call's spread with whole
+// lines, which sp becomes where memory is short, or the stream is being captured,
+// and only these fit: splitting is no reason to refuse a call.
+fqsl_status take_scratch(fqsl_field f, Spread &sp, const Spread &whole, long long n, bool rot, bool lattice, bool f32,
+                         bool m2, cudaStream_t stream, Scratch &s)
+{
+    const size_t want = scratch_bytes(sp, n, rot, lattice, f32, m2);
+    const size_t least = layout(nullptr, n, rot, lattice, f32, m2, false).bytes;
+    if (want > f->scratch_cap && least <= f->scratch_cap) {
+        // whole lines fit: grow only if that can be had, keeping what there is until then
+        void *more = nullptr;
+        if (!capturing(stream) && dev_malloc(&more, want) == cudaSuccess) {
+            const cudaError_t e = cudaDeviceSynchronize();
+            if (e != cudaSuccess) {
+                cudaFree(more);
+                return cuda_fail(e, "scratch: synchronize");
+            }
+            cudaFree(f->scratch);
+            f->scratch = more;
+            f->scratch_cap = want;
+        } else {
+            cudaGetLastError();
+        }
+    } else if (want > f->scratch_cap) {
+        fqsl_status st = ensure_scratch(f, want);
+        if (st == FQSL_ERR_OOM && least < want) {
+            g_err.clear();
+            st = ensure_scratch(f, least);
+        }
+        if (st != FQSL_OK) return st;
+    }
+    if (layout(nullptr, n, rot, lattice, f32, m2, sp.split).bytes > f->scratch_cap) sp = whole;
+    s = layout((char *)f->scratch, n, rot, lattice, f32, m2, sp.split);
     return FQSL_OK;
 }
 
@@ -1128,14 +1178,16 @@ fqsl_status run_qmap_locked(fqsl_field f, const Lattice &lat0, const fqsl_params
     const bool m2 = p->method == 2;
     const bool rot = lat.allow_rot != 0;
     Scratch s;
-    Spread sp{};
+    Spread sp{}, whole{};
     TapeLayout tl{};
     if (!tape) {
         const bool lane = line_per_lane(f, p, lat, face_plane);
         const int bps = m2 ? blocks_per_sm_m2(f, p)
                            : (lane ? lane_blocks_per_sm(f, p->scheme) : blocks_per_sm(f, p->precision, kSrcLattice, p->scheme));
-        sp = spread_of(f, p, lane ? 1 : lanes_per_line(p), bps, n, face_plane ? kSeedsFace : kSeedsInside,
-                       sparse_lattice(f->g, lat), true);
+        const int per = lane ? 1 : lanes_per_line(p);
+        const SeedKind kind = face_plane ? kSeedsFace : kSeedsInside;
+        sp = spread_of(f, p, per, bps, n, kind, sparse_lattice(f->g, lat), true);
+        whole = spread_of(f, p, per, bps, n, kind, sparse_lattice(f->g, lat), false);
     }
     if (tape) {
         tape->valid = false;
@@ -1159,9 +1211,8 @@ fqsl_status run_qmap_locked(fqsl_field f, const Lattice &lat0, const fqsl_params
         tl = tape_layout_of(tape, (char *)tape->buf, tape->pool);
         s = tl.s;
     } else {
-        fqsl_status st = ensure_scratch(f, scratch_bytes(sp, n, rot, true, f32, m2));
+        fqsl_status st = take_scratch(f, sp, whole, n, rot, true, f32, m2, stream, s);
         if (st != FQSL_OK) return st;
-        s = layout((char *)f->scratch, n, rot, true, f32, m2, sp.split);
     }
 
     cudaError_t e = cudaMemsetAsync(s.ctr, 0, s.zero_bytes, stream);
@@ -1438,11 +1489,12 @@ fqsl_status fqsl_twist(fqsl_field f, const double *seeds_dev, long long n, const
     cudaStream_t stream = (cudaStream_t)cuda_stream;
     const bool f32 = p->precision != FQSL_F64;
     std::lock_guard<std::mutex> lock(f->mu);
-    const Spread sp = spread_of(f, p, lanes_per_line(p), blocks_per_sm(f, p->precision, kSrcList, p->scheme), n,
-                                kSeedsList, true, true);
-    st = ensure_scratch(f, scratch_bytes(sp, n, false, false, f32, false));
+    const int bps = blocks_per_sm(f, p->precision, kSrcList, p->scheme);
+    Spread sp = spread_of(f, p, lanes_per_line(p), bps, n, kSeedsList, true, true);
+    const Spread whole = spread_of(f, p, lanes_per_line(p), bps, n, kSeedsList, true, false);
+    Scratch s;
+    st = take_scratch(f, sp, whole, n, false, false, f32, false, stream, s);
     if (st != FQSL_OK) return st;
-    Scratch s = layout((char *)f->scratch, n, false, false, f32, false, sp.split);
     cudaError_t e = cudaMemsetAsync(s.ctr, 0, s.zero_bytes, stream);
     if (e != cudaSuccess) return cuda_fail(e, who);
     TraceArgs a{};
