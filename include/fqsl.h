@@ -98,8 +98,9 @@ typedef struct {
     int gradb_way;        /* Method II gradient of B/|B|: 1 = node grid (Eq. grad_B), 2 = +-eps differences */
     int precision;        /* FQSL_F32 (default), FQSL_F64 or FQSL_F32_ACC64 (see fqsl_dtype) */
     int refill_lanes;     /* scheduling: a warp takes new seeds once this many of its 32 lanes are idle
-                             (1..32; 0 = library default; the FP64 tracer of Method I, which gives a line
-                             eight lanes, refills at once). Results do not depend on it. */
+                             (1..32; 0 = library default; the FP64 tracer of Method I refills at once where
+                             it gives a line eight lanes, which is all but very large planes). Results do
+                             not depend on it. */
     double tol;           /* tol_perp (Method I; scaled per line by |Bn0/B|^tol_exp) or tol (Method II, twist); default 10^-3.2 */
     double h0;            /* initial step, default 0.5 */
     double h_min;         /* smallest step, default 1e-6 */
@@ -110,11 +111,11 @@ typedef struct {
     double graze;         /* smallest outward face-normal velocity of the exit step, default 1e-3 */
     double eps_way2;      /* Method II way-2 offset, default 1e-3 */
     int sync_dirs;        /* scheduling: 1 = the lanes of a warp start their second directions together,
-                             0 = each lane at once, -1 = library default; FP64 Method I: at once. Results
-                             do not depend on it. */
+                             0 = each lane at once, -1 = library default; with eight lanes a line: at
+                             once. Results do not depend on it. */
     int chunk_tiles;      /* scheduling: 8x4-seed tiles a warp takes per grab of the work counter
                              (1..64; 0 = default: 1, or part of one where the lines do not fill the GPU;
-                             batches and FP64 Method I take at most 1). Results do not depend on it. */
+                             batches and lines of eight lanes take at most 1). Results do not depend on it. */
     int blocks_per_sm;    /* scheduling: resident 128-thread blocks per SM of the persistent tracer
                              (0 = library default: as many as fit, fewer for scattered seeds in a large
                              cube). Results do not depend on it. */
@@ -271,8 +272,8 @@ FQSL_API fqsl_status fqsl_twist(fqsl_field field, const double *seeds_dev, long 
  * records CUDA events on its own stream around its kernels; fqsl_field_times
  * waits for the events of the last call and returns their durations in
  * milliseconds: ms[0] line tracer (lattice or seed list; the FP32 seed
- * pre-pass runs just before it and is not included), ms[1] tracer of the
- * rotated-S0 extra lines (0 if not launched; a timed FP32 call gives them a
+ * pre-pass runs just before it and is not included), ms[1] set-up and tracer of
+ * the rotated-S0 extra lines (0 if not launched; a timed FP32 call gives them a
  * launch of their own, an untimed one traces them with the lattice), ms[2] Q
  * assembly. Errors:
  * FQSL_ERR_ARG (NULL, or no timed call yet), FQSL_ERR_CUDA. */

@@ -958,7 +958,8 @@ cudaError_t launch_trace(const fqsl_params *p, const TraceArgs &a, const Spread 
 }
 
 // The extra lines of rotated seeds in a launch of their own: the FP32 lattice
-// kernel with no lattice items, the FP64 one's own source.
+// kernel with no lattice items behind the lines' set-up, the FP64 one's own source
+// (which sets them up).
 cudaError_t launch_extra(fqsl_field f, const fqsl_params *p, TraceArgs a, const Scratch &s, Spread sp,
                          cudaStream_t stream)
 {
@@ -973,6 +974,8 @@ cudaError_t launch_extra(fqsl_field f, const fqsl_params *p, TraceArgs a, const 
     if (f32) {
         a.nitems = 0;
         a.p.merge = 1;
+        const cudaError_t e = launch_extra_prep_f32(a, stream);
+        if (e != cudaSuccess) return e;
     }
     return launch_trace(p, a, sp, f32 ? kSrcLattice : kSrcExtra, spread_grid(sp, f->sms, 0, true), stream);
 }
@@ -1248,7 +1251,7 @@ fqsl_status run_qmap_locked(fqsl_field f, const Lattice &lat0, const fqsl_params
     a.p.merge = !tape && f32 && rot && !f->timing;
     if (f32) {
         e = launch_seed_prep_f32(a, n, stream);
-        if (e == cudaSuccess && rot && !tape) e = launch_extra_prep_f32(a, stream);
+        if (e == cudaSuccess && a.p.merge) e = launch_extra_prep_f32(a, stream);
         if (e != cudaSuccess) return cuda_fail(e, who);
     }
     mark(f, 0, stream);
@@ -1665,7 +1668,7 @@ extern "C" fqsl_status fqsl_qmap_plane_static(fqsl_field f, const double origin[
     a.p.merge = f32 && rot && !f->timing;
     if (f32) {
         e = launch_seed_prep_f32(a, n, stream);
-        if (e == cudaSuccess && rot) e = launch_extra_prep_f32(a, stream);
+        if (e == cudaSuccess && a.p.merge) e = launch_extra_prep_f32(a, stream);
         if (e != cudaSuccess) return cuda_fail(e, who);
     }
     mark(f, 0, stream);
