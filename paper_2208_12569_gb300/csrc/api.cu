@@ -86,8 +86,7 @@ struct fqsl_field_s {
     void *scratch = nullptr;
     size_t scratch_cap = 0;
     void *rect_buf = nullptr;  // stretched grid: coordinate, width and bucket tables (FieldView::x64 ...)
-    unsigned long long *counters = nullptr;  // [0] primary head, [1] extra head, [2] rotated count (low 32 bits),
-                                             // [4] first failed index check of the adjoint kernels, [5] their count
+    unsigned long long *counters = nullptr;  // [4] first failed index check of the adjoint kernels, [5] their count
     int blocks_cache[2][3][3] = {};  // [scheme][precision][source] resident blocks per SM
     int blocks_cache_lane[2] = {};   // FP64 lattices with a lane per line: [scheme]
     int blocks_cache_m2[2][2][2] = {};  // Method II: [scheme][fp64][way - 1]

@@ -1,6 +1,6 @@
-// Persistent field-line tracer (templated on the traced precision T; the FP64
-// maps of Method I and seed lists are traced by trace64.cuh, in the arithmetic
-// that this file states).
+// Persistent field-line tracer (templated on the traced precision T; FP64 maps
+// of Method I and seed lists are traced by trace64.cuh, in the arithmetic that
+// this file states, but for very large planes: trace64_lane.cu).
 //
 // Method (Zhang et al. 2022):
 //   - field-line equation dr/ds = B/|B| (Sec. 2.1, Eq. rb), integrated in index
@@ -47,6 +47,12 @@
 // against 23.4 ms, smaller maps up to 1.2 times as long at 6 and 8.
 #ifndef FQSL_TRACE_F64_MINB
 #define FQSL_TRACE_F64_MINB 4
+#endif
+
+// Resident blocks per SM asked of the FP32 Method II tracers: 3 (168 registers, a
+// few spills); 2 measured slower (384x256 seeds, way 2: 2.90 against 2.77 ms)
+#ifndef FQSL_TRACE_DEV_F32_MINB
+#define FQSL_TRACE_DEV_F32_MINB 3
 #endif
 
 namespace fqsl {
@@ -852,7 +858,7 @@ __device__ __forceinline__ bool unit_b(const FieldView &f, T x, T y, T z, T bh[3
 }
 
 // dd: the trial's per-axis scale (step_dd): on a stretched grid way 2 offsets
-// +-eps cells of the start cell, eps D_a (FP64 dd = D, FP32 dd = 1/D).
+// +-eps cells of the start cell, eps D_a. (Way 2 in FP32: grad_way2_32.)
 template <typename T, int WAY, bool RECT = false>
 __device__ __forceinline__ bool grad_bhat(const FieldView &f, T eps, T x, T y, T z, const T dd[3], T G[3][3])
 {
@@ -861,6 +867,7 @@ __device__ __forceinline__ bool grad_bhat(const FieldView &f, T eps, T x, T y, T
         else gather_grad(f, x, y, z, G);
         return true;
     } else {
+        static_assert(sizeof(T) == 8, "FP64");
         const T p[3] = {x, y, z};
         bool ok = true;
 #pragma unroll
@@ -868,9 +875,8 @@ __device__ __forceinline__ bool grad_bhat(const FieldView &f, T eps, T x, T y, T
             T xp[3] = {p[0], p[1], p[2]}, xm[3] = {p[0], p[1], p[2]};
             T off = eps, span;
             if constexpr (RECT) {
-                const T D = sizeof(T) == 8 ? dd[a] : (T)1 / dd[a];
-                off = eps * D;
-                span = (T)2 * eps * D;
+                off = eps * dd[a];
+                span = (T)2 * eps * dd[a];
             } else {
                 span = (T)2 * eps * (T)f.d[a];
             }
@@ -1145,7 +1151,8 @@ __device__ __forceinline__ void write_end32(const LineRecs &R, long long line, i
 }
 
 // ---------------------------------------------------------------------------
-// step tape (adjoint forward pass; see Tape)
+// step tape (adjoint forward pass; see Tape) of the FP32 tracer; the double stores
+// are the reverse sweep's
 // ---------------------------------------------------------------------------
 // 16-byte vector stores of the kept states and stage derivatives (addresses
 // 16-byte aligned: the arrays are, and their strides are multiples of 16 B).
@@ -1238,11 +1245,10 @@ __device__ __forceinline__ void tape_end(const Tape &tp, Lane<T> &L, int code, T
 }
 
 // Split directions (the taped tracer): each direction of a line is its own
-// work item, so the line's status bits, trial count and (FP64) length/Tw sums
-// are combined with atomics on records cleared before the launch. Each
-// direction finishes with its share; the one that completes the trial count
-// marks the line MAXSTEPS if both together used more than max_steps. (A sum of
-// two values onto zero does not depend on their order.)
+// work item, so the line's status bits and trial count are combined with atomics
+// on records cleared before the launch. Each direction finishes with its share;
+// the one that completes the trial count marks the line MAXSTEPS if both together
+// used more than max_steps.
 __device__ __forceinline__ void or_status(uint8_t *st, long long line, unsigned bits)
 {
     unsigned *w = (unsigned *)(st + (line & ~3LL));
@@ -1631,19 +1637,12 @@ __device__ __forceinline__ bool init_lattice(const TraceArgs &A, Lane<T> &L, lon
     const FieldView &f = A.f;
     const LineRecs &R = A.rec;
     if constexpr (!kF64) return load_seed<T, ACC, DEV>(A, L, idx);
-    double xi[3];
-    if (kF64) {
-        // physical seed, then (r0 - o)/d, as written (the physical seed itself
-        // on a stretched grid)
-        double r0[3];
-        lattice_seed(G, i, j, k, r0);
+    // physical seed, then (r0 - o)/d, as written (the physical seed itself on a
+    // stretched grid)
+    double xi[3], r0[3];
+    lattice_seed(G, i, j, k, r0);
 #pragma unroll
-        for (int a = 0; a < 3; a++) xi[a] = state_of<T, RECT>(f, r0[a], a);
-    } else {
-        const double fi = (double)i + 0.5, fj = (double)j + 0.5, fk = (double)k + 0.5;
-#pragma unroll
-        for (int a = 0; a < 3; a++) xi[a] = fma(fk, G.xa3[a], fma(fj, G.xa2[a], fma(fi, G.xa1[a], G.xo[a])));
-    }
+    for (int a = 0; a < 3; a++) xi[a] = state_of<T, RECT>(f, r0[a], a);
     // B at the seed, S0 obliquity and tolerance (fixed-step scheme: step)
     double tol = ctl_perp(A.p);
     int st0 = 0;
@@ -1674,15 +1673,8 @@ __device__ __forceinline__ bool init_lattice(const TraceArgs &A, Lane<T> &L, lon
                     }
                 } else {
                     bn0 = (double)bn;
-                    if (A.p.scheme == 1) {
-                        tol = fmax(A.p.step * (double)ratio, A.p.step_min);  // Eq. step
-                    } else if (kF64) {
-                        tol = A.p.tol * obliq_pow(fmax((double)ratio, A.p.rot), A.p.texp);
-                    } else {
-                        const float x = fmaxf((float)ratio, (float)A.p.rot);
-                        const float g = A.p.texp == 1.5 ? x * sqrtf(x) : __powf(x, (float)A.p.texp);
-                        tol = A.p.tol * (double)g;
-                    }
+                    if (A.p.scheme == 1) tol = fmax(A.p.step * (double)ratio, A.p.step_min);  // Eq. step
+                    else tol = A.p.tol * obliq_pow(fmax((double)ratio, A.p.rot), A.p.texp);
                 }
             }
         }

@@ -5,12 +5,6 @@
 // per-line tolerance, footpoints and Bn are double in both.
 #include "trace.cuh"
 
-// resident blocks per SM asked of the Method II tracers: 3 (168 registers, a few
-// spills); 2 measured slower (384x256 seeds, way 2: 2.90 against 2.77 ms)
-#ifndef FQSL_TRACE_DEV_F32_MINB
-#define FQSL_TRACE_DEV_F32_MINB 3
-#endif
-
 // minimum resident blocks per SM requested from the register allocator
 #ifndef FQSL_TRACE_F32_MINB
 #define FQSL_TRACE_F32_MINB 4
@@ -52,7 +46,8 @@ int blocks(int src)
 
 cudaError_t launch_trace_f32(const TraceArgs &a, int src, int grid, int block, cudaStream_t s, bool acc64)
 {
-    if (block != kBlock) return cudaErrorInvalidValue;
+    // (extra lines follow the lattice's items: DevParams::merge)
+    if (block != kBlock || src == kSrcExtra) return cudaErrorInvalidValue;
     if (a.p.scheme == 1)
         return a.f.rect ? launch_trace_rect_rk38_f32(a, src, grid, s, acc64) : launch_trace_rk38_f32(a, src, grid, s, acc64);
     if (a.f.rect) return launch_trace_rect_f32(a, src, grid, s, acc64);

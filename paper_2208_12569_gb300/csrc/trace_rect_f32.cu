@@ -5,12 +5,6 @@
 // Method II's deviation vectors), plus the FP32 seed pre-pass on such a grid.
 #include "trace.cuh"
 
-// resident blocks per SM asked of the Method II tracers: 3 (168 registers, a few
-// spills); 2 measured slower (384x256 seeds, way 2: 2.90 against 2.77 ms)
-#ifndef FQSL_TRACE_DEV_F32_MINB
-#define FQSL_TRACE_DEV_F32_MINB 3
-#endif
-
 #ifndef FQSL_TRACE_F32_MINB
 #define FQSL_TRACE_F32_MINB 4
 #endif

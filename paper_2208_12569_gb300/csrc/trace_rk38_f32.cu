@@ -6,12 +6,6 @@
 // tracers of the adjoint's forward pass.
 #include "trace.cuh"
 
-// resident blocks per SM asked of the Method II tracers: 3 (168 registers, a few
-// spills); 2 measured slower (384x256 seeds, way 2: 2.90 against 2.77 ms)
-#ifndef FQSL_TRACE_DEV_F32_MINB
-#define FQSL_TRACE_DEV_F32_MINB 3
-#endif
-
 #ifndef FQSL_TRACE_F32_MINB
 #define FQSL_TRACE_F32_MINB 4
 #endif
