@@ -1077,6 +1077,7 @@ struct Lane {
 // lane came by the line.
 constexpr int kLaneExtra = 0x100;  // an extra line of a rotated seed (no length/Tw sums are kept)
 constexpr int kLaneSplit = 0x200;  // the line's other direction is another lane's (see split_join)
+constexpr int kLaneAsked = 0x400;  // and, from here up, how often it was asked whether that is done (split_steps)
 
 // Length and Tw of the current direction: FP64 sums (ACC, and the FP64
 // tracer) or compensated FP32 sums (Kahan 1965) whose total is formed in FP64
@@ -1286,6 +1287,26 @@ __device__ __forceinline__ void start_second(const TraceArgs &A, Lane<T> &L)
     acc_reset<T, ACC>(L);
 }
 
+// A second direction of a split line counts its trials up to max_steps from
+// split_ask_every below it, and again each time it gets there (kLaneAsked: how
+// often), so that the hot loop's one comparison also stops it to ask for the
+// first direction (a test of its own there cost small maps and lists 2 to 3 %).
+__device__ __forceinline__ int split_ask_every(int max_steps) { return max(128, max_steps >> 20); }
+
+template <typename T>
+__device__ __forceinline__ void split_second(const TraceArgs &A, Lane<T> &L)
+{
+    L.end = 1;
+    L.steps = max((int)A.p.max_steps - split_ask_every((int)A.p.max_steps), 0);
+}
+
+// The trials that a second direction's count stands for.
+__device__ __forceinline__ int split_steps(int max_steps, int steps, int st)
+{
+    const int every = split_ask_every(max_steps);
+    return steps - max(max_steps - every, 0) + (st / kLaneAsked) * every;
+}
+
 // Untaped maps too small to fill the GPU give the two directions of a line to
 // two lanes (kLaneSplit; FP32). Each lane adds its trial count (bits 0-31), its
 // status (bits 32-39 and 40-47) and how it ended (48, 49: done; 50, 51: bad)
@@ -1294,12 +1315,13 @@ __device__ __forceinline__ void start_second(const TraceArgs &A, Lane<T> &L)
 // ends the line (end 2 is the seed, only the first direction's trials count),
 // and if both together reach max_steps the second direction is traced again
 // with what the first left of the budget (a second direction that outlives the
-// first has joined it before, see split_adopt). Returns whether this lane has to.
+// first has joined it before, see split_goes_on). Returns whether this lane has to.
 template <typename T, bool ACC, int DEV>
 __device__ __forceinline__ bool split_join(const TraceArgs &A, const LineRecs &R, Lane<T> &L, bool bad)
 {
-    if (L.end == 0) *(volatile int32_t *)(R.steps + L.line) = L.steps;
-    const unsigned long long mine = (unsigned long long)(unsigned)L.steps |
+    const int steps = L.end ? split_steps((int)A.p.max_steps, L.steps, L.st) : L.steps;
+    if (L.end == 0) *(volatile int32_t *)(R.steps + L.line) = steps;
+    const unsigned long long mine = (unsigned long long)(unsigned)steps |
                                     ((unsigned long long)((unsigned)L.st & 0xffu) << (32 + 8 * L.end)) |
                                     (1ull << (48 + L.end)) | ((bad ? 1ull : 0ull) << (50 + L.end));
     __threadfence();  // this direction's end record, before the other lane can see it as done
@@ -1325,39 +1347,26 @@ __device__ __forceinline__ bool split_join(const TraceArgs &A, const LineRecs &R
     return false;
 }
 
-// The second direction of a split line, 128 trials after it last asked: is the
-// first one done? Then this lane takes the line over as one that traced both
-// directions, the first one's trials and status included, so that a line that
-// runs into max_steps does so with its whole budget known. (Left to split_join such
-// a line was traced twice: a volume of 64x64x32 seeds of a 512x512x128 cube whose
-// longest line is trapped, 425 ms; with this 209.)
-__device__ __forceinline__ bool split_first_done(const LineRecs &R, long long line)
+// The second direction of a split line is out of steps, or has done another
+// split_ask_every of them. In the latter case, if the first direction is done,
+// its lane takes the line over as one that traced both directions, the first
+// one's trials and status included, so that a line that runs into max_steps does
+// so with its whole budget known. (Left to split_join such a line was traced
+// twice: a volume of 64x64x32 seeds of a 512x512x128 cube whose longest line is
+// trapped, 425 ms; with this 209.) Returns {steps, st} to go on with, or a negative
+// steps if the direction ends here: out of steps, or of the line's, or behind a bad
+// first one (split_join sorts that out). Out of line and by value: inlined it cost
+// the hot loop of lists 1 % more.
+static __device__ __noinline__ int2 split_goes_on(const unsigned long long *pair, int steps, int st, int max_steps)
 {
-    return (*(volatile unsigned long long *)(R.pair + line) >> 48) & 1ull;
-}
-
-// Returns whether the lane goes on (its position may be the seed again).
-template <typename T, bool ACC, int DEV>
-__device__ __forceinline__ bool split_adopt(const TraceArgs &A, const LineRecs &R, Lane<T> &L)
-{
+    const int done = split_steps(max_steps, steps, st);
+    if (done >= max_steps) return make_int2(-1, 0);
+    const unsigned long long w = *(volatile const unsigned long long *)pair;
+    if (!((w >> 48) & 1ull)) return make_int2(steps - split_ask_every(max_steps), st + kLaneAsked);
     __threadfence();
-    const unsigned long long w = *(volatile unsigned long long *)(R.pair + L.line);
-    const int st0 = (int)(w >> 32) & 0xff;
-    const int32_t steps0 = *(volatile int32_t *)(R.steps + L.line);
-    if ((w >> 50) & 1ull) {
-        write_end32(R, L.line, 1, (float)L.sx, (float)L.sy, (float)L.sz, -1);
-        R.st[L.line] = (uint8_t)st0;
-        return false;
-    }
-    if ((long long)steps0 + L.steps > A.p.max_steps) {
-        L.st = st0 | (L.st & kLaneExtra);
-        L.steps = steps0;
-        start_second<T, ACC, DEV>(A, L);
-        return true;
-    }
-    L.st = (L.st & ~kLaneSplit) | st0;
-    L.steps += steps0;
-    return true;
+    const long long both = (long long)(w & 0xffffffffull) + done;  // (the word holds the first one's trials)
+    if (((w >> 50) & 1ull) || both > max_steps) return make_int2(-1, 0);
+    return make_int2((int)both, (st & (0xff | kLaneExtra)) | ((int)(w >> 32) & 0xff));
 }
 
 // Finish the line with a bad status (MAXSTEPS or NULL_B): the unfinished end
@@ -1391,6 +1400,23 @@ __device__ __forceinline__ bool finish_bad(const TraceArgs &A, const LineRecs &R
         R.steps[L.line] = L.steps;
     }
     return false;
+}
+
+// L.steps has reached max_steps. Returns whether the lane goes on.
+template <typename T, bool ACC, int DEV, bool SPLIT, bool RECT, bool FLEX>
+__device__ __forceinline__ bool out_of_steps(const TraceArgs &A, const LineRecs &R, Lane<T> &L)
+{
+    if constexpr (FLEX) {
+        if ((L.st & kLaneSplit) && L.end == 1) {
+            const int2 next = split_goes_on(R.pair + L.line, L.steps, L.st, (int)A.p.max_steps);
+            if (next.x >= 0) {
+                L.steps = next.x;
+                L.st = next.y;
+                return true;
+            }
+        }
+    }
+    return finish_bad<T, ACC, DEV, SPLIT, RECT, FLEX>(A, R, L, FQSL_LINE_MAXSTEPS);
 }
 
 // A direction reached a face at index position (x, y, z) with deviation
@@ -1772,7 +1798,7 @@ template <typename T, int SRC, bool ACC, int DEV = 0, bool BATCH = false, bool T
           int SCH = 0, bool FLEX = false>
 __device__ __forceinline__ void trace_body(const TraceArgs &A0, const BatchArgs &BA)
 {
-    if constexpr (SRC == kSrcList) {
+    if constexpr (SRC == kSrcList && !FLEX) {  // (lists that are split are short)
         if (A0.q.blocks && blockIdx.x >= *A0.q.blocks) return;
     }
     constexpr bool SPLIT = TAPE && SRC == kSrcLattice;
@@ -1801,7 +1827,7 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A0, const BatchArgs 
     // lines: with them the lines may fill more lanes (48x48 seeds, all rotated:
     // 0.52 ms with the lattice's two lanes, 0.22 with sixteen).
     int take = A0.p.lanes;
-    if (MERGED && A0.p.merge)
+    if (MERGED && !BATCH && A0.p.merge)
         while (take < 32 && nitems > (long long)gridDim.x * (blockDim.x / 32) * take) take *= 2;
     const unsigned gmask = take >= 32 ? FULL : (1u << take) - 1u;
 
@@ -1828,7 +1854,7 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A0, const BatchArgs 
             if (ck_cur >= ck_end) {
                 unsigned long long base = 0;
                 // (at most 32 with BATCH or p.split)
-                const long long chunk = MERGED && A0.p.lanes < 32 ? __popc(gmask) : A0.p.chunk;
+                const long long chunk = MERGED && !BATCH && A0.p.lanes < 32 ? __popc(gmask) : A0.p.chunk;
                 if (lane == 0) base = atomicAdd(A0.q.head, (unsigned long long)chunk);
                 base = __shfl_sync(FULL, base, 0);
                 if ((long long)base >= nitems) {
@@ -1881,7 +1907,7 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A0, const BatchArgs 
                         }
                         if (FLEX && active) {
                             L.st |= fl;
-                            if (psplit && ((item >> 5) & 1)) L.end = 1;
+                            if (psplit && ((item >> 5) & 1)) split_second(A0, L);
                         }
                     }
                 } else if constexpr (SRC == kSrcExtra) {
@@ -1892,7 +1918,7 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A0, const BatchArgs 
                     active = slot < nlat && init_list<T, ACC, RECT>(E, L, slot);
                     if (active && psplit) {
                         L.st |= kLaneSplit;
-                        if ((item >> 5) & 1) L.end = 1;
+                        if ((item >> 5) & 1) split_second(A0, L);
                     }
                 }
             }
@@ -1929,14 +1955,8 @@ __device__ __forceinline__ void trace_body(const TraceArgs &A0, const BatchArgs 
         const T sgn = (L.end == 0) ? -L.s0 : L.s0;
         T hh;
         if (!henon) {
-            if constexpr (FLEX) {
-                if ((L.steps & 127) == 127 && (L.st & kLaneSplit) && L.end == 1 && split_first_done(R, L.line)) {
-                    active = split_adopt<T, ACC, DEV>(A, R, L);
-                    continue;
-                }
-            }
             if (L.steps >= max_steps) {
-                active = finish_bad<T, ACC, DEV, SPLIT, RECT, FLEX>(A, R, L, FQSL_LINE_MAXSTEPS);
+                active = out_of_steps<T, ACC, DEV, SPLIT, RECT, FLEX>(A, R, L);
                 continue;
             }
             hh = L.h;
