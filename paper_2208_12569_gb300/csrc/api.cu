@@ -609,8 +609,8 @@ enum SeedKind {
     kSeedsList     // an explicit list: whether neighbours in it are neighbours in space is seen on the device
 };
 
-// Blocks per SM. FP32 lines that share no cells (lists; lattices two cells
-// apart) touch pages of the node records all over a large cube, and more
+// Blocks per SM. FP32 lines that share few cells (lists; lattices 1.5 cells apart)
+// touch pages of the node records all over a large cube, and more
 // resident lanes than the address translation can serve make each load slower
 // than they hide: nothing but the latency is busy (ncu, 2.1 GB of records, 4
 // blocks: L1 24 %, L2 19 %, DRAM 25 %; 2 blocks are 1.4 times as fast with the
@@ -622,14 +622,15 @@ enum SeedKind {
 //   1.44 GB  14.22 /  9.20 / 10.70          9.96 /  8.67 /  7.17
 //   2.15 GB  20.01 / 11.83 / 12.49         12.19 / 10.58 /  8.53
 // (a plane of 1024x512 seeds half a cell apart in the last cube: 5.43 / 5.86 / 7.40).
-// Lattices a given number of cells apart, at 4 / 3 blocks (1.34 GB; 2.0 GB):
-//   cells  plane inside               volume
-//   0.9    2.15 / 2.53; 2.67 / 3.09   0.87 / 0.95; 3.11 / 3.27
-//   1      2.24 / 2.56; 2.68 / 3.12   1.02 / 1.10; 3.45 / 3.58
-//   1.4    2.10 / 2.30; 2.98 / 3.15   1.86 / 1.91; 4.17 / 4.20
-//   2      2.11 / 1.80; 2.61 / 2.68   3.56 / 3.36; 4.19 / 3.80
-//   4      1.25 / 1.17; 2.01 / 1.71   6.24 / 4.17; 5.37 / 3.85
-// A list may hold a plane's or a curve's seeds in order. list_blocks (trace_f32.cu)
+// Lattices a given number of cells apart, time at 3 blocks over that at 4:
+//   cells   1.3 GB: bottom / plane inside / volumes   4 GB                        16 GB
+//   1       1.08 / 1.11 / 1.06-1.09                   1.06 / 1.10 / 1.03-1.07     0.89 / 1.04 / 1.03-1.07
+//   1.25    1.05 / 1.06 / 1.05-1.07                   1.00 / 1.07 / 1.01-1.05     0.78 / 0.85 / 1.01-1.04
+//   1.5     0.98 / 0.88 / 1.04-1.06                   0.86 / 1.00 / 1.01-1.03     0.77 / 0.71 / 0.97-1.01
+//   1.75    0.89 / 0.86 / 0.99-1.00                   0.69 / 0.87 / 0.94-0.97     0.80 / 0.64 / 0.74-0.94
+//   2       0.94 / 0.82 / 0.88-0.90                   0.67 / 0.79 / 0.80          0.82 / 0.71 / 0.56-0.73
+//   2.5     0.85 / 0.75 / 0.75-0.76                   0.77 / 0.65 / 0.55-0.60     0.88 / 0.76 / 0.53-0.65
+// A list may hold a plane's or a curve's seeds in order. k_list_blocks (trace_f32.cu)
 // looks at pairs of neighbours spread over the list and holds it to the fewer
 // blocks only if most are more than 1.5 cells apart. Rows of 300,000 seeds, ms at 4 /
 // 3 / 2 blocks (the last column with 2 cells shuffled):
@@ -638,12 +639,11 @@ enum SeedKind {
 //   0.85 GB   1.69 / 1.82 / 2.25   1.81 / 1.64 / 2.01   3.26 / 2.44 / 2.62   4.88 / 4.12 / 4.05
 //   1.34 GB   1.44 / 1.59 / 1.99   1.71 / 1.65 / 2.08   3.38 / 2.35 / 2.37   5.32 / 4.48 / 4.21
 //   2.00 GB   1.32 / 1.47 / 1.85   1.80 / 1.97 / 2.46   2.90 / 2.02 / 2.26   5.57 / 4.67 / 4.49
-int tlb_blocks(size_t record_bytes, SeedKind kind, bool sparse, int bps)
+int tlb_blocks(size_t record_bytes, SeedKind kind, double apart, int bps)
 {
-    if (!sparse) return bps;
     int most = bps;
     if (kind == kSeedsList) most = record_bytes >= ((size_t)700 << 20) ? 2 : (record_bytes >= ((size_t)400 << 20) ? 3 : bps);
-    else if (record_bytes >= ((size_t)1200 << 20)) most = 3;
+    else if (record_bytes >= ((size_t)1200 << 20) && apart >= (record_bytes >= ((size_t)8 << 30) ? 1.25 : 1.5)) most = 3;
     return most < bps ? most : bps;
 }
 
@@ -697,14 +697,14 @@ bool line_per_lane(const fqsl_field f, const fqsl_params *p, const Lattice &lat,
     return n >= (p->scheme == 0 && face ? 8 : 6) * full;
 }
 
-Spread spread_of(const fqsl_field f, const fqsl_params *p, int per, int bps, long long lines, SeedKind kind, bool sparse,
+Spread spread_of(const fqsl_field f, const fqsl_params *p, int per, int bps, long long lines, SeedKind kind, double apart,
                  bool may_split)
 {
     const bool f32 = p->precision != FQSL_F64;
     Spread r{bps, per, 32, 0, false, 0};
     int blocks = bps;  // blocks whose lanes the lines are spread over
     if (p->blocks_per_sm > 0) blocks = p->blocks_per_sm < bps ? p->blocks_per_sm : bps;
-    else if (f32 && lines > (long long)f->sms * kTraceBlock) blocks = tlb_blocks((size_t)f->g.nodes * 32, kind, sparse, bps);
+    else if (f32 && lines > (long long)f->sms * kTraceBlock) blocks = tlb_blocks((size_t)f->g.nodes * 32, kind, apart, bps);
     if (kind == kSeedsList && p->blocks_per_sm <= 0 && blocks < bps) r.few = blocks;
     else r.bps = blocks;
     const long long warps = (long long)f->sms * blocks * (kTraceBlock / 32);
@@ -732,9 +732,9 @@ int tape_lanes(const fqsl_params *p, long long warps, long long items)
     return lanes;
 }
 
-// Are a lattice's seeds two cells or more apart (its 8x4-seed tile covers at
-// least four times as many cells as it has seeds)?
-bool sparse_lattice(const FieldView &g, const Lattice &lat)
+// How many cells a lattice's seeds are apart (the root of the cells that its
+// 8x4-seed tile covers per seed).
+double cells_apart(const FieldView &g, const Lattice &lat)
 {
     double area = 1.0;
     const double *step[2] = {lat.a1, lat.a2};
@@ -747,7 +747,7 @@ bool sparse_lattice(const FieldView &g, const Lattice &lat)
         }
         area *= s;
     }
-    return area >= 4.0;
+    return sqrt(area);
 }
 
 struct Scratch {
@@ -1188,8 +1188,8 @@ fqsl_status run_qmap_locked(fqsl_field f, const Lattice &lat0, const fqsl_params
                            : (lane ? lane_blocks_per_sm(f, p->scheme) : blocks_per_sm(f, p->precision, kSrcLattice, p->scheme));
         const int per = lane ? 1 : lanes_per_line(p);
         const SeedKind kind = face_plane ? kSeedsFace : kSeedsInside;
-        sp = spread_of(f, p, per, bps, n, kind, sparse_lattice(f->g, lat), true);
-        whole = spread_of(f, p, per, bps, n, kind, sparse_lattice(f->g, lat), false);
+        sp = spread_of(f, p, per, bps, n, kind, cells_apart(f->g, lat), true);
+        whole = spread_of(f, p, per, bps, n, kind, cells_apart(f->g, lat), false);
     }
     if (tape) {
         tape->valid = false;
@@ -1492,8 +1492,8 @@ fqsl_status fqsl_twist(fqsl_field f, const double *seeds_dev, long long n, const
     const bool f32 = p->precision != FQSL_F64;
     std::lock_guard<std::mutex> lock(f->mu);
     const int bps = blocks_per_sm(f, p->precision, kSrcList, p->scheme);
-    Spread sp = spread_of(f, p, lanes_per_line(p), bps, n, kSeedsList, true, true);
-    const Spread whole = spread_of(f, p, lanes_per_line(p), bps, n, kSeedsList, true, false);
+    Spread sp = spread_of(f, p, lanes_per_line(p), bps, n, kSeedsList, 0.0, true);
+    const Spread whole = spread_of(f, p, lanes_per_line(p), bps, n, kSeedsList, 0.0, false);
     Scratch s;
     st = take_scratch(f, sp, whole, n, false, false, f32, false, stream, s);
     if (st != FQSL_OK) return st;
@@ -1634,12 +1634,12 @@ extern "C" fqsl_status fqsl_qmap_plane_static(fqsl_field f, const double origin[
     const bool rot = lat.allow_rot != 0;
     std::lock_guard<std::mutex> lock(f->mu);
     const SeedKind kind = face_plane ? kSeedsFace : kSeedsInside;
-    const bool sparse = sparse_lattice(f->g, lat);
+    const double apart = cells_apart(f->g, lat);
     const int bps = blocks_per_sm(f, p->precision, kSrcLattice, p->scheme);
-    Spread sp = spread_of(f, p, lanes_per_line(p), bps, n, kind, sparse, true);
+    Spread sp = spread_of(f, p, lanes_per_line(p), bps, n, kind, apart, true);
     Scratch need = layout(nullptr, n, rot, true, f32, false, sp.split);
     if (need.bytes > kStaticScratchBytes && sp.split) {
-        sp = spread_of(f, p, lanes_per_line(p), bps, n, kind, sparse, false);
+        sp = spread_of(f, p, lanes_per_line(p), bps, n, kind, apart, false);
         need = layout(nullptr, n, rot, true, f32);
     }
     if (need.bytes > kStaticScratchBytes)

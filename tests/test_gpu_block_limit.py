@@ -1,7 +1,7 @@
 """FP32 launches over a large cube hold fewer resident blocks only where their
-lines share no cells. Seeds a cell apart share them: such a call may not be
+lines share few cells. Seeds a cell apart share them: such a call may not be
 slower than with as many blocks as fit (a sixteenth is allowed for noise), and
-seeds four cells apart may not either."""
+neither may seeds four cells apart. A plane two cells apart has to be faster."""
 import pytest
 import torch
 
@@ -43,9 +43,9 @@ def _calls(fq, call):
     return [lambda p=fq.params(precision="f32", blocks_per_sm=b): call(p) for b in (0, 8)]
 
 
-@pytest.mark.parametrize("apart", [1.0, 1.3, 4.0])
-@pytest.mark.parametrize("shape", ["plane", "volume"])
-def test_lattice(field, apart, shape):
+@pytest.mark.parametrize("shape,apart", [("plane", 1.0), ("plane", 1.3), ("plane", 1.99), ("plane", 4.0), ("volume", 1.0),
+                                         ("volume", 1.3), ("volume", 4.0)])
+def test_lattice(field, shape, apart):
     fq, f = field
     w, h = min(800, int((N[0] - 2) / apart)), min(500, int((N[1] - 2) / apart))
     if shape == "plane":
@@ -60,7 +60,7 @@ def test_lattice(field, apart, shape):
         def call(p):
             fq.qmap_volume(f, (0.2, 0.2, 0.2), (apart,) * 3, w, h, d, p=p, out=out)
     limited, free = _ms(_calls(fq, call))
-    assert limited < 1.0625 * free, (limited, free)
+    assert limited < (0.97 if apart == 1.99 else 1.0625) * free, (limited, free)
 
 
 def _rows(apart):
