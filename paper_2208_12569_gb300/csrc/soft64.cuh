@@ -110,22 +110,40 @@ FQSL_HD float rsqrt_approx(float x)
 #endif
 }
 
-// the hardware operations, for operands outside the integer paths' range
-#ifdef __CUDA_ARCH__
-static __device__ __noinline__ double hw_div(double a, double b) { return __ddiv_rn(a, b); }
-static __device__ __noinline__ double hw_sqrt(double a) { return __dsqrt_rn(a); }
-static __device__ __forceinline__ double hw_mul(double a, double b) { return __dmul_rn(a, b); }
-#else
-static inline double hw_div(double a, double b) { return a / b; }
-static inline double hw_sqrt(double a) { return sqrt(a); }
-static inline double hw_mul(double a, double b) { return a * b; }
-#endif
-
 constexpr uint32_t kExpMask = 0x7ff00000u;
 constexpr uint32_t kExpLow = 768u << 20;  // smallest exponent field of the integer paths
 
 // 0 where the exponent field e (in place) is in range, else one of the top 3 bits set
 FQSL_HD uint32_t out_of_range(uint32_t e) { return (e - kExpLow) & 0xe0000000u; }
+
+// Operands outside the integer paths' range: the hardware operations, but for
+// exact zeros over a divisor in range and under the root. Those are ordinary (a
+// component of a field along an axis, J of a current-free one, the error of a
+// straight line's step), and sent to the hardware they made a lane of each group
+// wait for the FP64 pipe beside the others' integer quotients: FP64 map of 512x512
+// seeds in a constant field of an anisotropic 128x128x64 cube 38.0 ms, 20.8 with
+// this; gradient grid of a vertical field 256x128x64 2.0 ms, 0.55. (Out of line: the
+// test in every quotient cost the gradient grid 3 %.)
+#ifdef __CUDA_ARCH__
+#define FQSL_OUTSIDE static __device__ __noinline__
+static __device__ __forceinline__ double hw_div(double a, double b) { return __ddiv_rn(a, b); }
+static __device__ __forceinline__ double hw_sqrt(double a) { return __dsqrt_rn(a); }
+static __device__ __forceinline__ double hw_mul(double a, double b) { return __dmul_rn(a, b); }
+#else
+#define FQSL_OUTSIDE static inline
+static inline double hw_div(double a, double b) { return a / b; }
+static inline double hw_sqrt(double a) { return sqrt(a); }
+static inline double hw_mul(double a, double b) { return a * b; }
+#endif
+
+FQSL_OUTSIDE double div_outside(double a, double b)
+{
+    const uint32_t ah = (uint32_t)(bits_of(a) >> 32), bh = (uint32_t)(bits_of(b) >> 32);
+    if (!(bits_of(a) << 1) && !out_of_range(bh & kExpMask)) return of_words((ah ^ bh) & 0x80000000u, 0u);
+    return hw_div(a, b);
+}
+
+FQSL_OUTSIDE double sqrt_outside(double x) { return bits_of(x) << 1 ? hw_sqrt(x) : x; }
 
 // Round the 53-bit integer m (its leading bit set) with the fraction word r
 // (units of 2^-32, its low bits sticky) to nearest, ties to even, and pack it
@@ -255,19 +273,9 @@ FQSL_HD double div_in_range(double x, const Divisor &d)
     return round_pack(q >> 4, r, e, (h & 0x80000000u) ^ d.s);
 }
 
-// (Exact zeros are ordinary here: a component of a field along an axis, J of a
-// current-free one, the error of a straight line's step. Sent to the hardware
-// they made a lane of each group wait for the FP64 pipe beside the others'
-// integer quotients: FP64 map of 512x512 seeds in a constant field of an
-// anisotropic 128x128x64 cube 38.0 ms, 20.1 with this; gradient grid of a vertical
-// field 256x128x64 2.0 ms, 0.57.)
 FQSL_HD double div64(double a, const Divisor &d)
 {
-    const uint64_t b = bits_of(a);
-    if (d.bad | out_of_range((uint32_t)(b >> 32) & kExpMask)) {
-        if (!d.bad && !(b << 1)) return of_words(((uint32_t)(b >> 32) & 0x80000000u) ^ d.s, 0u);
-        return hw_div(a, d.x);
-    }
+    if (d.bad | out_of_range((uint32_t)(bits_of(a) >> 32) & kExpMask)) return div_outside(a, d.x);
     return div_in_range(a, d);
 }
 
@@ -277,7 +285,7 @@ FQSL_HD double sqrt64(double x)
 {
     const uint64_t b = bits_of(x);
     const uint32_t h = (uint32_t)(b >> 32);
-    if (out_of_range(h)) return (b << 1) ? hw_sqrt(x) : x;  // (a set sign bit is out of range too)
+    if (out_of_range(h)) return sqrt_outside(x);  // (a set sign bit is out of range too)
     // x = m 2^(2k - 52) with m / 2^52 in [1, 4)
     const uint32_t odd = ((h >> 20) & 1u) ^ 1u;  // (exponent less 1023) odd
     const uint64_t m = ((b & 0xfffffffffffffull) | (1ull << 52)) << odd;
