@@ -656,16 +656,22 @@ int tlb_blocks(size_t record_bytes, SeedKind kind, double apart, int bps)
 //     of a 88x66x50 cube 0.57 -> 0.66 ms), and a list so
 //     short that every direction gets a warp of its own (a longer list gains
 //     nothing: 8,000 seeds 0.456 ms either way, 30,000 0.61 against 0.54 ms).
+//     Maps and volumes of 16,000 to 230,000 seeds take 0.5 to 0.95 of the time with
+//     whole lines; lines that are all alike gain nothing and pay (65,536 seeds in a
+//     nearly uniform field 0.32 -> 0.41 ms, vertical cuts of 100,000 to 230,000
+//     seeds of a 128x128x64 stretched cube up to 1.12 times). Limits of 56, 40 and 24
+//     times the warps for 96 lost 10 to 25 % on volumes and horizontal planes.
 //     Not a lattice on a box face, where one direction ends at once and its
 //     lanes would idle (90,000 seeds 0.62 -> 1.17 ms).
 //   lanes: fewer lines per warp until the lines fill the resident warps: lanes
 //     of one warp whose lines have parted wait for each other's loads (list of
 //     500 seeds 0.36 -> 0.26 ms with 2 lanes, plane of 4,096 seeds 0.38 -> 0.32
 //     ms with 4; with more warps than fit at once it loses: 90,000 seeds of a
-//     plane 0.62 -> 0.84 ms, a list of 40,604 seeds 0.45 -> 0.56 ms). Whole lines, one after the other, are spread less
-//     below 16 lanes: 8,000 seeds of a list in a 64x64x64 cube 0.160 ms with 8
-//     lanes and 0.177 with 4, 128x128 seeds of its bottom 0.287 ms with 16, 0.295
-//     with 8 and 0.290 with 32. The FP64 tracer of Method I gives a line eight
+//     plane 0.62 -> 0.84 ms, a list of 40,604 seeds 0.45 -> 0.56 ms). Whole lines,
+//     one after the other, are spread less below 16 lanes: 8,000 seeds of a list in
+//     a 64x64x64 cube 0.160 ms with 8 lanes and 0.177 with 4, 128x128 seeds of its
+//     bottom 0.287 ms with 16, 0.295 with 8 and 0.290 with 32. Extra lines, which
+//     only the device can count, widen the lanes there. The FP64 tracer of Method I gives a line eight
 //     lanes, so four lines fill a warp. FP64 Method II lines, one per lane, are
 //     spread only over SMs that would idle: their warp instructions take the
 //     narrow FP64 pipe the same time whatever their lanes.

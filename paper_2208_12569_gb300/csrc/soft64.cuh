@@ -8,16 +8,18 @@
 // products: a quotient in about 100 issue slots (fewer when the divisor is
 // shared) and a square root in about 110, each of which holds the FP64 pipe
 // for about ten instructions, 640 cycles, as hardware code. The FP64 tracer
-// with these two: 25.5 ms for a map of 512x512 seeds, 33.2 ms with the
-// hardware's. The multiply, about 35 slots, is correct too but loses to the
-// pipe's 64 cycles there (trace64.cuh).
+// with these two, and with the hardware's: 21.5 and 33.0 ms for a map of 512x512
+// seeds, 80.8 and 126 ms for 1024x1024; four updates of a 256x256x128 gradient
+// grid 6.2 and 15.5 ms. The multiply, about 35 slots, is correct too but loses to
+// the pipe's 64 cycles in the tracer (trace64.cuh) and is used by nothing.
 //
 // The integer paths take operands with biased exponents in [768, 1279], that
 // is 2^-255 <= |x| < 2^257, whose results can neither overflow nor be
 // subnormal, and a zero divided by such a divisor or under the root; anything
 // else (subnormals, infinities, NaNs, huge and tiny values) goes to the hardware
-// operation. Both give the same bits, so which one runs shows in no result. All of it compiles for the host as well, where
-// a test compares it with the processor's own operations.
+// operation. Both give the same bits, so which one runs shows in no result. All
+// of it compiles for the host as well, where a test compares it with the
+// processor's own operations.
 //
 // Methods: schoolbook products of 32-bit digits; quotient digits from a
 // truncated reciprocal with an exact remainder (long division in base 2^28,

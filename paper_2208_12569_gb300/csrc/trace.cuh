@@ -41,10 +41,10 @@
 
 #include "fqsl_internal.cuh"
 
-// Resident 128-thread blocks per SM asked of the FP64 tracers of Method I
-// (trace64.cuh; about 100 registers a lane): 4. At 3, 5, 6 and 8 blocks a map of
-// 512x512 seeds of the 256x256x128 cube took 23.5, 23.6, 25.3 and 25.4 ms
-// against 23.4 ms, smaller maps up to 1.2 times as long at 6 and 8.
+// Resident 128-thread blocks per SM asked of the FP64 tracers that give a line
+// eight lanes (trace64.cuh; about 100 registers a lane): 4. At 3, 5, 6 and 8 blocks
+// a map of 512x512 seeds of the 256x256x128 cube took 23.5, 23.6, 25.3 and 25.4 ms
+// against 23.4 ms at 4, smaller maps up to 1.2 times as long at 6 and 8.
 #ifndef FQSL_TRACE_F64_MINB
 #define FQSL_TRACE_F64_MINB 4
 #endif

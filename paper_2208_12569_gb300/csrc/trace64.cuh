@@ -19,15 +19,15 @@
 // for four lines at once. Divisions and square roots, about ten FP64
 // instructions each, run on the integer pipe (soft64.cuh); products and sums
 // stay on the FP64 pipe (products on the integer pipe too: 35.1 ms against 25.5
-// ms for the 512x512 map below, half of the gather's 27.2 ms: 30 issue slots
-// and an instruction cache that runs out cost more than 64 cycles of a pipe
-// that other warps leave idle).
+// ms for a map of 512x512 seeds in an earlier build, half of the gather's 27.2
+// ms: 30 issue slots and an instruction cache that runs out cost more than 64
+// cycles of a pipe that other warps leave idle).
 //
-// Measured against the line-per-lane form (256x256x128 cube unless noted,
-// outputs bit-identical): bottom plane of 512x512 seeds 33.5 -> 23.4 ms (FP64
-// pipe 75 % busy), of 1024x1024 91.2 -> 78.4 ms, vertical cut of 700x512 102.5 ->
-// 78.3 ms, a list of 400,000 seeds 123 -> 55.7 ms and of 3,801 (182x124x144 cube)
-// 5.6 -> 2.1 ms.
+// Measured against the line-per-lane form (256x256x128 cube, outputs
+// bit-identical; spacing 1 / anisotropic / stretched, ms): bottom plane of
+// 512x512 seeds 31.0 -> 21.5 / 30.4 -> 23.0 / 44.2 -> 35.9 (FP64 pipe 76 % busy), of
+// 1024x1024 94.9 -> 80.8 / 91.4 -> 87.0 / 143 -> 139, a list of 400,000 seeds 135 ->
+// 66.5 / 157 -> 84.1 / 196 -> 105. Larger planes: api.cu, line_per_lane.
 #pragma once
 
 #include "soft64.cuh"
